@@ -4,26 +4,25 @@
 // Sec. III-C) behind a virtual leader whose gap dp_k and speed difference
 // dv_k at every step are free variables.
 //
-// One thread per trajectory, one warp per block.  Every per-step array is
-// time-major, so at step k a warp touches one 128-byte row segment per array.
+// One thread per trajectory.  Every per-step array is time-major, so at step k
+// a warp touches one 128-byte row segment per array.  The simulation, the loss
+// gradient and the metrics run one warp per block (recon_kernel); the fit, whose
+// iterations repeat the same trajectories hundreds of times, splits 32
+// trajectories' steps over the warps of a block (recon_fit_kernel, below).
 // Rows are staged into shared memory with cp.async, S - 1 chunks of U steps
 // ahead of use, so the forward's serial chain (the speed of step k+1 needs the
 // whole model evaluation of step k) does not wait on memory: rows of the
 // caller's arrays with 16-byte copies shared by the warp (then __syncwarp), or
 // with 4-byte copies of each lane's own column when the row stride is not a
-// multiple of four; the tape and the Adam moments with one 16-byte copy per
-// lane of its own data.
+// multiple of four; the tape with one 16-byte copy per lane of its own data.
 //
-// Forward: integrates the state and, while its serial chain (one model
-// evaluation per step) leaves most issue slots idle, evaluates the adjoint's
-// partials of every step (they depend only on the step's speed, dp_k and dv_k)
-// and writes them with the loss seed of step k+1 as the tape; or writes the
-// requested P/V/A, or the metric sums.  Adjoint: walks the tape backwards; its
-// only serial chain is the adjoint recursion (two FMAs per step), the rest
-// (gradient sums, Adam on dp_k and dv_k) is independent across steps.  The fit
-// runs every iteration of its trajectory inside one launch (trajectories are
-// independent), with Adam for dp_k and dv_k fused into the adjoint and Adam
-// for the parameters at its end.
+// recon_kernel's forward: integrates the state and, while its serial chain (one
+// model evaluation per step) leaves most issue slots idle, evaluates the
+// adjoint's partials of every step (they depend only on the step's speed, dp_k
+// and dv_k) and writes them with the loss seed of step k+1 as the tape; or
+// writes the requested P/V/A, or the metric sums.  Its adjoint walks the tape
+// backwards; its only serial chain is the adjoint recursion (two FMAs per step),
+// the rest is independent across steps.
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdint.h>
@@ -45,12 +44,12 @@ constexpr int U = 8;                       // steps per staged chunk
 constexpr int S = 3;                       // chunks in flight
 // A stage holds, per step and lane: three float4 slots (forward: the rows of
 // dp, dv, the observed position and the observation code, overlaid as four
-// float rows; adjoint: the two tape halves and the Adam moments or the delta
-// factor) and two float rows (adjoint: dp, dv).
+// float rows; adjoint: the two tape halves and the delta factor) and two float
+// rows (adjoint: dp, dv).
 constexpr int STAGE = (3 * 4 + 2) * U * 32;   // floats per chunk
 constexpr int SMEM = (int)sizeof(float) * S * STAGE;
 
-enum Mode { FWD_OUT = 0, LOSS_GRAD = 1, FIT = 2, METRICS = 3 };
+enum Mode { FWD_OUT = 0, LOSS_GRAD = 1, METRICS = 2 };
 
 struct Args {
     int N, k_max, ld, n_obs;
@@ -67,6 +66,7 @@ struct Args {
     const float *obs_p;
     float4 *tape_a, *tape_b;         // tape [k_max][ld]: (Av, Adp, Adv, w0n), (w0n v, fa, frd, seed of step k+1)
     float *tape_d;                   // [k_max][ld]: frdl (delta gradient only)
+    float *tape_v, *tape_s;          // fit: [k_max][ld] speed of step k, seed of step k+1
     float4 *mom;                     // [k_max][ld]: Adam moments (m_dp, v_dp, m_dv, v_dv)
     float *thm, *thv;                // Adam moments of the parameters, [5][N]
     float *P, *V, *A;
@@ -306,12 +306,12 @@ struct MetricAcc {
 };
 
 // Forward over the Ki steps of trajectory i (Kw = the warp's largest Ki).
-// Returns the loss sum (LOSS_GRAD, FIT), which also write the tape.
+// Returns the loss sum (LOSS_GRAD, which also writes the tape).
 template <int MODE, bool D4, bool WD>
 __device__ __forceinline__ double fwd_phase(const Args &a, const Par &q, int i, bool act, int Ki, int Kw, float *sm,
                                             int lane, MetricAcc &ma, float len_inv)
 {
-    constexpr bool TAPE = MODE == LOSS_GRAD || MODE == FIT;
+    constexpr bool TAPE = MODE == LOSS_GRAD;
     const int nch = (Kw + U - 1) / U;
     const size_t ld = (size_t)a.ld;
     const int i0 = i - lane;
@@ -337,7 +337,7 @@ __device__ __forceinline__ double fwd_phase(const Args &a, const Par &q, int i, 
     float ph = act ? a.p_init[i] : 0.0f, pl = 0.0f;
     float Ls = 0.0f, Lcomp = 0.0f;   // loss: per-thread Kahan sum of the chunk sums
     const int j_end =
-        (MODE == LOSS_GRAD || MODE == FIT || MODE == METRICS) && Ki > 0 ? min(a.obs_off[i + 1], a.n_obs) : 0;
+        (MODE == LOSS_GRAD || MODE == METRICS) && Ki > 0 ? min(a.obs_off[i + 1], a.n_obs) : 0;
     // One chunk of U steps.  MULTI: some step of the chunk has several
     // observations (rare); without it the chunk is one branch-free block, so
     // the compiler can overlap a step's partials, position and observation
@@ -457,9 +457,9 @@ __device__ __forceinline__ float adam1(float x, float g, float &m, float &w, flo
 // of step k+1 enters lambda_p before step k is reversed.  Returns the
 // parameter sums A[6] (gradients assembled by the caller), lambda_p(0) and
 // lambda_v(0).
-template <int MODE, bool WD>
-__device__ __forceinline__ void adj_phase(const Args &a, int i, int Ki, int Kw, float *sm, int lane, float a1,
-                                          float isb2, float (&Acc)[6], float &lp_out, float &lv_out)
+template <bool WD>
+__device__ __forceinline__ void adj_phase(const Args &a, int i, int Ki, int Kw, float *sm, int lane, float (&Acc)[6],
+                                          float &lp_out, float &lv_out)
 {
     const int nch = (Kw + U - 1) / U;
     const size_t ld = (size_t)a.ld;
@@ -474,7 +474,6 @@ __device__ __forceinline__ void adj_phase(const Args &a, int i, int Ki, int Kw, 
                     const size_t o = (size_t)k * ld + i;
                     cp16(slot4(sm, c, 0, u, lane), a.tape_a + o);
                     cp16(slot4(sm, c, 1, u, lane), a.tape_b + o);
-                    if (MODE == FIT) cp16(slot4(sm, c, 2, u, lane), a.mom + o);
                     if (WD) cp4(reinterpret_cast<float *>(slot4(sm, c, 2, u, lane)), a.tape_d + o);
                 }
             }
@@ -516,19 +515,8 @@ __device__ __forceinline__ void adj_phase(const Args &a, int i, int Ki, int Kw, 
             lp = valid ? lpn : lp;
             lv = valid ? lvn : lv;
             const size_t o = (size_t)k * ld + i;
-            if (MODE == LOSS_GRAD) {
-                if (valid && a.g_dp) a.g_dp[o] = gdp;
-                if (valid && a.g_dv) a.g_dv[o] = gdv;
-            } else if (MODE == FIT) {
-                float4 m = *slot4(sm, c, 2, u, lane);
-                const float dpn = adam1(pv.x, gdp, m.x, m.y, a1, isb2);
-                const float dvn = adam1(pv.y, gdv, m.z, m.w, a1, isb2);
-                if (valid) {
-                    a.dp[o] = dpn;
-                    a.dv[o] = dvn;
-                    a.mom[o] = m;
-                }
-            }
+            if (valid && a.g_dp) a.g_dp[o] = gdp;
+            if (valid && a.g_dv) a.g_dv[o] = gdv;
         }
     }
     cp_wait<0>();
@@ -605,9 +593,9 @@ __device__ __forceinline__ void run_single(const Args &a, int i, bool act, int K
         __threadfence_block();  // the tape written above is read back by this thread's copies
         float A[6], lp, lv, gr[6];
         if (wd)
-            adj_phase<LOSS_GRAD, true>(a, i, Ki, Kw, sm, lane, 0.0f, 0.0f, A, lp, lv);
+            adj_phase<true>(a, i, Ki, Kw, sm, lane, A, lp, lv);
         else
-            adj_phase<LOSS_GRAD, false>(a, i, Ki, Kw, sm, lane, 0.0f, 0.0f, A, lp, lv);
+            adj_phase<false>(a, i, Ki, Kw, sm, lane, A, lp, lv);
         if (!act) return;
         param_grads(q, A, gr);
         bool bad = !isfinite(lp) || !isfinite(lv);
@@ -643,63 +631,388 @@ __global__ void __launch_bounds__(32) recon_kernel(Args a)
         run_single<MODE, false>(a, i, act, Ki, Kw, sm, lane);
 }
 
-// The whole fit of every trajectory of the warp: n_iter x {forward with the
-// loss and seeds, adjoint with Adam on dp and dv, Adam on the parameters}.
-template <bool D4>
-__device__ __forceinline__ void fit_warp(const Args &a, int i, bool act, int Ki, int Kw, float *sm, int lane)
+// ---- the fit --------------------------------------------------------------------
+// n_iter x {forward with the loss and seeds, adjoint with Adam on dp and dv,
+// Adam on the parameters} of 32 trajectories per block, one launch.
+//
+// What bounds it: the forward's serial chain (the speed of step k+1 needs the
+// whole model at step k: ~105 cycles of dependent latency), and how much of a
+// step's other work (positions and observations, the adjoint's partials, the
+// gradient sums, Adam on dp and dv, the copies) runs beside it.  One warp
+// doing all of it spends ~640 cycles per step on its own instruction stream,
+// so the block's warps split a step by role, pipelined over chunks of CH steps
+// with one block barrier per chunk (a tick).  Warps 0 and 1 run the serial
+// chains and the ordered sums, each of NW workers everything of SPW steps of a
+// chunk:
+//   forward, tick t:  warp 0 the speeds of chunk t; warp 1 the positions of
+//     chunk t - 1 and the loss sum of chunk t - 3; the workers the residual, the
+//     seed and the tape (speed and seed, 8 bytes) of their steps of chunk t - 2;
+//   adjoint, tick t:  the workers the partials of their steps of chunk t, from
+//     the taped speed, and Adam on dp and dv of their steps of chunk t - 2; warp
+//     0 the recursion and two parameter sums of chunk t - 1; warp 1 the other
+//     three of chunk t - 2.
+// Each worker stages the rows and moments of its steps D chunks ahead.  Every
+// sum keeps one owner and its order, so a trajectory's result does not depend
+// on the split.  With the partials evaluated beside the recursion instead of
+// taped by the forward, a trajectory-step moves 80 bytes instead of 128.
+namespace fit {
+constexpr int CH = 16, NW = 8, SPW = CH / NW;
+constexpr int W = 2 + NW;        // warps per block
+constexpr int ROW = CH * 32;     // floats of one staged array of a chunk
+// Shared floats.  Adjoint: rows (dp, dv, speed, seed; D + 3 chunks in flight
+// and in use), moments (D + 1), the partial Av of the recursion and the factors
+// fa, frd of its sums (2), w0n (3), mu (2).  The forward's rows (dp, dv,
+// observed position and code), speeds (3), position pairs (2) and absolute
+// residuals (2) lie over them.
+template <int D>
+struct Lay {
+    static constexpr int R = D + 3, RM = D + 1;
+    static constexpr int O_MOM = R * 4 * ROW, O_AV = O_MOM + RM * 4 * ROW, O_W0 = O_AV + 2 * 3 * ROW, O_MU = O_W0 + 3 * ROW;
+    static constexpr int O_TH = O_MU + 2 * ROW, FLOATS = O_TH + 5 * 32;
+    static constexpr int O_V = R * 4 * ROW, O_P = O_V + 3 * ROW, O_R = O_P + 2 * 2 * ROW;
+    static_assert(O_R + 2 * ROW <= O_TH, "the forward's stages lie below the parameters");
+    static constexpr int BYTES = (int)sizeof(float) * FLOATS;
+};
+}  // namespace fit
+
+// Stage step k's rows of four arrays into rows[(r CH + u) 32 + column]: one
+// 16-byte copy per lane (wide: array lane / 8, segment lane % 8 of the 128-byte
+// row; needs ld % 4 == 0, 16-byte aligned arrays, i0 + 32 <= ld; src_l = that
+// array + i0 + 4 (lane % 8)), or four 4-byte copies of the lane's own column.
+__device__ __forceinline__ void fit_stage(float *rows, const float *const (&src)[4], const float *src_l, size_t ld, int i,
+                                          int lane, int u, int k, bool wide, bool own)
 {
+    if (wide) {
+        cp16(rows + ((lane >> 3) * fit::CH + u) * 32 + (lane & 7) * 4, src_l + (size_t)k * ld);
+    } else if (own) {
+#pragma unroll
+        for (int r = 0; r < 4; ++r) cp4(rows + (r * fit::CH + u) * 32 + lane, src[r] + (size_t)k * ld + i);
+    }
+}
+__device__ __forceinline__ const float *fit_lane_src(const float *const (&src)[4], int i0, int lane)
+{
+    const int r = lane >> 3;
+    return (r < 2 ? (r == 0 ? src[0] : src[1]) : (r == 2 ? src[2] : src[3])) + i0 + (lane & 7) * 4;
+}
+
+// Forward of one iteration; returns the loss of this lane's trajectory in warp 1.
+template <bool D4, int D>
+__device__ __forceinline__ double fit_forward(const Args &a, const Par &q, int i, bool act, int Ki, int Kw, bool multi,
+                                              bool wide, float *sm, int lane, int w)
+{
+    using L = fit::Lay<D>;
+    using fit::CH;
+    using fit::ROW;
+    const int nch = (Kw + CH - 1) / CH;
+    const size_t ld = (size_t)a.ld;
+    const int u0 = w - 2;   // the worker's steps: u0 + NW h
+    const float *const src[4] = {a.dp, a.dv, a.oyy, reinterpret_cast<const float *>(a.oyc)};
+    const float *const src_l = fit_lane_src(src, i - lane, lane);
+    auto rows = [&](int c) { return sm + (size_t)(c % L::R) * 4 * ROW; };
+    auto speeds = [&](int c) { return sm + L::O_V + (c % 3) * ROW + lane; };
+    auto pairs = [&](int c) { return reinterpret_cast<float2 *>(sm + L::O_P) + (c & 1) * ROW + lane; };
+    auto absres = [&](int c) { return sm + L::O_R + (c & 1) * ROW + lane; };
+    auto issue = [&](int c) {
+#pragma unroll
+        for (int h = 0; h < fit::SPW; ++h) {
+            const int u = u0 + fit::NW * h, k = c * CH + u;
+            if (k < Kw) fit_stage(rows(c), src, src_l, ld, i, lane, u, k, wide, k < Ki);
+        }
+        cp_commit();
+    };
+    const float dt = a.dt, inv_dt = a.inv_dt, a_min = a.a_min;
+    float v = act ? a.v_init[i] : 0.0f;
+    float ph = act ? a.p_init[i] : 0.0f, pl = 0.0f;
+    float Ls = 0.0f, Lcomp = 0.0f;   // loss: Kahan sum of the sums of eight steps
+    const int j_end = Ki > 0 ? min(a.obs_off[i + 1], a.n_obs) : 0;
+    if (w >= 2) {
+#pragma unroll
+        for (int c = 0; c < D; ++c) issue(c);
+        cp_wait<D - 1>();
+    }
+    __syncthreads();
+    for (int t = 0; t < nch + 3; ++t) {
+        if (w >= 2) {
+            issue(t + D);
+            const int c = t - 2;
+            if (c >= 0) {
+                const float *rw = rows(c) + 2 * ROW + lane, *vw = speeds(c);
+                const float2 *pw = pairs(c);
+                float *aw = absres(c);
+#pragma unroll
+                for (int h = 0; h < fit::SPW; ++h) {
+                    const int u = u0 + fit::NW * h, k = c * CH + u;
+                    const float2 pos = pw[u * 32];   // after step k
+                    const float vk = vw[u * 32];
+                    // observations at step k+1: the staged first one, then
+                    // (multi) any further ones from the CSR
+                    const int code = k < Ki ? __float_as_int(rw[ROW + u * 32]) : -1;
+                    const bool has = code >= 0;
+                    float r = (pos.x - rw[u * 32]) + pos.y;
+                    float seed = has ? sgn(r) : 0.0f;
+                    float sum = has ? fabsf(r) : 0.0f;
+                    if (multi && has && (code & 7) > 1) {
+                        const int cnt = code & 7, j0 = code >> 3;
+                        for (int j = j0 + 1; j < j_end; ++j) {
+                            if (cnt < 7 ? j >= j0 + cnt : a.obs_k[j] != k + 1) break;
+                            r = (pos.x - a.obs_p[j]) + pos.y;
+                            seed += sgn(r);
+                            sum += fabsf(r);
+                        }
+                    }
+                    aw[u * 32] = sum;
+                    if (k < Ki) {
+                        const size_t o = (size_t)k * ld + i;
+                        a.tape_v[o] = vk;
+                        a.tape_s[o] = seed;
+                    }
+                }
+            }
+            cp_wait<D - 1>();
+        } else if (w == 0) {
+            if (t < nch) {
+                const float *rw = rows(t) + lane;
+                float *vw = speeds(t);
+#pragma unroll
+                for (int s = 0; s < CH; ++s) {
+                    const float dp = rw[s * 32], dv = rw[ROW + s * 32];
+                    const float gap_inv = rcp_approx(fmaxf(dp, IDM_GAP_FLOOR));
+                    float as;
+                    const float vn = speed_step<D4>(v, gap_inv, fmaf(dv, q.c, q.T), q, dt, inv_dt, a_min, as);
+                    vw[s * 32] = v;
+                    v = t * CH + s < Ki ? vn : v;
+                }
+            }
+        } else {
+            const int c = t - 1;
+            if (c >= 0 && c < nch) {
+                const float *vw = speeds(c);
+                float2 *pw = pairs(c);
+#pragma unroll
+                for (int s = 0; s < CH; ++s) {
+                    float phn = ph, pln = pl;
+                    euler_pos(phn, pln, vw[s * 32], dt);
+                    const bool valid = c * CH + s < Ki;
+                    ph = valid ? phn : ph;
+                    pl = valid ? pln : pl;
+                    pw[s * 32] = make_float2(ph, pl);
+                }
+            }
+            if (t >= 3) {
+                const float *rs = absres(t - 3);
+#pragma unroll
+                for (int g = 0; g < CH; g += 8) {
+                    float Lc = 0.0f;
+#pragma unroll
+                    for (int s = g; s < g + 8; ++s) Lc += rs[s * 32];
+                    kahan(Ls, Lcomp, Lc);
+                }
+            }
+        }
+        __syncthreads();
+    }
+    if ((w == 0 && !isfinite(v)) || (w == 1 && !isfinite(ph + pl))) atomicOr(a.status, IDM_STATUS_NONFINITE);
+    return (double)Ls - (double)Lcomp;
+}
+
+// Adjoint of one iteration with Adam on dp and dv (first: the moments are
+// still zero).  Of the parameter sums, 3 and 4 end in warp 0, the others in
+// warp 1.
+template <bool D4, int D>
+__device__ __forceinline__ void fit_adjoint(const Args &a, const Par &q, int i, int Ki, int Kw, bool wide, float *sm,
+                                            int lane, int w, float a1, float isb2, bool first, float (&Acc)[6])
+{
+    using L = fit::Lay<D>;
+    using fit::CH;
+    using fit::ROW;
+    const int nch = (Kw + CH - 1) / CH;
+    const size_t ld = (size_t)a.ld;
+    const int u0 = w - 2;
+    const float *const src[4] = {a.dp, a.dv, a.tape_v, a.tape_s};
+    const float *const src_l = fit_lane_src(src, i - lane, lane);
+    auto rows = [&](int c) { return sm + (size_t)(c % L::R) * 4 * ROW; };
+    auto moms = [&](int c) { return reinterpret_cast<float4 *>(sm + L::O_MOM) + (c % L::RM) * ROW + lane; };
+    auto avs = [&](int c) { return sm + L::O_AV + (c & 1) * 3 * ROW + lane; };
+    auto w0s = [&](int c) { return sm + L::O_W0 + (c % 3) * ROW + lane; };
+    auto mus = [&](int c) { return sm + L::O_MU + (c & 1) * ROW + lane; };
+    auto step_of = [&](int c, int s) { return Kw - 1 - (c * CH + s); };
+    // rows of chunk c + 2 and moments of chunk c of the worker's steps
+    auto issue = [&](int c) {
+#pragma unroll
+        for (int h = 0; h < fit::SPW; ++h) {
+            const int u = u0 + fit::NW * h, k = step_of(c + 2, u), km = step_of(c, u);
+            if (k >= 0) fit_stage(rows(c + 2), src, src_l, ld, i, lane, u, k, wide, k < Ki);
+            if (!first && c >= 0 && km >= 0 && km < Ki) cp16(moms(c) + u * 32, a.mom + (size_t)km * ld + i);
+        }
+        cp_commit();
+    };
+    const float dt = a.dt;
+    float lp = 0.0f, lv = 0.0f;
+    float2 g1[fit::SPW], g2[fit::SPW];   // Adp, Adv of the worker's steps one and two chunks back
+#pragma unroll
+    for (int h = 0; h < fit::SPW; ++h) g1[h] = g2[h] = make_float2(0.0f, 0.0f);
+#pragma unroll
+    for (int r = 0; r < 6; ++r) Acc[r] = 0.0f;
+    if (w >= 2) {
+#pragma unroll
+        for (int c = 0; c < D; ++c) issue(c - 2);
+        cp_wait<D - 1>();
+    }
+    __syncthreads();
+    for (int t = 0; t < nch + 2; ++t) {
+        if (w >= 2) {
+            issue(t + D - 2);
+            float2 g3[fit::SPW];
+#pragma unroll
+            for (int h = 0; h < fit::SPW; ++h) {
+                g3[h] = g2[h];
+                g2[h] = g1[h];
+            }
+            if (t < nch) {
+                const float *rw = rows(t) + lane;
+                float *av = avs(t), *w0 = w0s(t);
+#pragma unroll
+                for (int h = 0; h < fit::SPW; ++h) {
+                    const int u = u0 + fit::NW * h;
+                    const Jac1 J = jac1<D4, false>(rw[2 * ROW + u * 32], rw[u * 32], rw[ROW + u * 32], q, a.inv_dt, a.a_min);
+                    av[u * 32] = J.Av;
+                    av[ROW + u * 32] = J.fa;
+                    av[2 * ROW + u * 32] = J.frd;
+                    w0[u * 32] = J.w0n;
+                    g1[h] = make_float2(J.Adp, J.Adv);
+                }
+            }
+            if (t >= 2) {
+                const float *rw = rows(t - 2) + lane, *mw = mus(t - 2);
+                const float4 *mo = moms(t - 2);
+#pragma unroll
+                for (int h = 0; h < fit::SPW; ++h) {
+                    const int u = u0 + fit::NW * h, k = step_of(t - 2, u);
+                    const float mu = mw[u * 32];
+                    float4 m = mo[u * 32];
+                    if (first) m = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+                    const float dpn = adam1(rw[u * 32], mu * g3[h].x, m.x, m.y, a1, isb2);
+                    const float dvn = adam1(rw[ROW + u * 32], mu * g3[h].y, m.z, m.w, a1, isb2);
+                    if (k >= 0 && k < Ki) {
+                        const size_t o = (size_t)k * ld + i;
+                        a.dp[o] = dpn;
+                        a.dv[o] = dvn;
+                        a.mom[o] = m;
+                    }
+                }
+            }
+            cp_wait<D - 1>();
+        } else if (w == 0) {
+            const int c = t - 1;
+            if (c >= 0 && c < nch) {
+                const float *rw = rows(c) + 3 * ROW + lane, *av = avs(c);
+                float *mw = mus(c);
+#pragma unroll
+                for (int s = 0; s < CH; ++s) {
+                    const int k = step_of(c, s);
+                    const bool valid = k >= 0 && k < Ki;
+                    const float lpn = lp + rw[s * 32];                           // lambda_p(k+1)
+                    const float mu = dt * lv;                                     // dt lambda_v(k+1)
+                    const float lvn = fmaf(mu, av[s * 32], fmaf(dt, lpn, lv));    // lambda_v(k)
+                    Acc[3] = valid ? fmaf(mu, av[ROW + s * 32], Acc[3]) : Acc[3];
+                    Acc[4] = valid ? fmaf(mu, av[2 * ROW + s * 32], Acc[4]) : Acc[4];
+                    mw[s * 32] = mu;
+                    lp = valid ? lpn : lp;
+                    lv = valid ? lvn : lv;
+                }
+            }
+        } else {
+            const int c = t - 2;
+            if (c >= 0) {
+                const float *rw = rows(c) + ROW + lane, *w0 = w0s(c), *mw = mus(c);
+#pragma unroll
+                for (int s = 0; s < CH; ++s) {
+                    const int k = step_of(c, s);
+                    const bool valid = k >= 0 && k < Ki;
+                    const float mu = mw[s * 32], w0n = w0[s * 32], w0nv = w0n * rw[ROW + s * 32];
+                    Acc[0] = valid ? fmaf(mu, w0n, Acc[0]) : Acc[0];
+                    Acc[1] = valid ? fmaf(mu, w0nv, Acc[1]) : Acc[1];
+                    Acc[2] = valid ? fmaf(mu, w0nv * rw[s * 32], Acc[2]) : Acc[2];
+                }
+            }
+        }
+        __syncthreads();
+    }
+}
+
+template <bool D4, int D>
+__device__ __forceinline__ void fit_block(const Args &a, int i, bool act, int Ki, int Kw, float *sm, int lane, int w)
+{
+    using L = fit::Lay<D>;
     Par q = act ? load_par(a, i) : make_par(1.0f, 1.0f, 1.0f, 1.0f, 1.0f, 4.0f);
     float th[5] = {q.v0, q.T, q.s0, q.am, q.b};
+    const bool multi = __any_sync(FULL, act && Ki > 0 && a.multi[i] != 0);   // several observations at one step
+    const bool wide = a.wide_ok && i - lane + 32 <= a.ld;                     // block-uniform
     bool bad = false;
-    MetricAcc ma;
     for (int it = 0; it < a.n_iter; ++it) {
-        const double L = fwd_phase<FIT, D4, false>(a, q, i, act, Ki, Kw, sm, lane, ma, 0.0f);
-        const double s = warp_sum(L);
-        if (lane == 0 && a.loss) atomicAdd(a.loss + it, s);
-        __threadfence_block();  // tape and updated dp, dv are read back by this thread's copies
+        const double loss = fit_forward<D4, D>(a, q, i, act, Ki, Kw, multi, wide, sm, lane, w);
+        if (w == 1) {
+            const double s = warp_sum(loss);
+            if (lane == 0 && a.loss) atomicAdd(a.loss + it, s);
+        }
         const int t = it + 1;
         const float lr = a.n_iter > 1 ? a.lr0 + (a.lr1 - a.lr0) * (float)it / (float)(a.n_iter - 1) : a.lr0;
         const float bc1 = 1.0f - __powf(0.9f, (float)t), bc2 = 1.0f - __powf(0.999f, (float)t);
         const float a1 = lr / bc1, isb2 = 1.0f / sqrtf(bc2);
-        float A[6], lp, lv, gr[6];
-        adj_phase<FIT, false>(a, i, Ki, Kw, sm, lane, a1, isb2, A, lp, lv);
-        __threadfence_block();
-        if (act) {
-            param_grads(q, A, gr);
+        float A[6], gr[6];
+        fit_adjoint<D4, D>(a, q, i, Ki, Kw, wide, sm, lane, w, a1, isb2, it == 0, A);
+        if (w == 0) {
+            sm[L::O_TH + lane] = A[3];
+            sm[L::O_TH + 32 + lane] = A[4];
+        }
+        __syncthreads();
+        if (w == 1) {
+            A[3] = sm[L::O_TH + lane];
+            A[4] = sm[L::O_TH + 32 + lane];
+            if (act) {
+                param_grads(q, A, gr);
 #pragma unroll
-            for (int r = 0; r < 5; ++r) {
-                bad |= !isfinite(gr[r]);
-                const size_t mi = (size_t)r * a.N + i;
-                const float m = 0.9f * a.thm[mi] + 0.1f * gr[r];
-                const float vv = 0.999f * a.thv[mi] + 0.001f * gr[r] * gr[r];
-                a.thm[mi] = m;
-                a.thv[mi] = vv;
-                const float x = th[r] - lr * (m / bc1) / (sqrtf(vv / bc2) + 1e-8f);
-                th[r] = fminf(fmaxf(x, a.lo[r]), a.hi[r]);
+                for (int r = 0; r < 5; ++r) {
+                    bad |= !isfinite(gr[r]);
+                    const size_t mi = (size_t)r * a.N + i;
+                    const float m = 0.9f * a.thm[mi] + 0.1f * gr[r];
+                    const float vv = 0.999f * a.thv[mi] + 0.001f * gr[r] * gr[r];
+                    a.thm[mi] = m;
+                    a.thv[mi] = vv;
+                    const float x = th[r] - lr * (m / bc1) / (sqrtf(vv / bc2) + 1e-8f);
+                    th[r] = fminf(fmaxf(x, a.lo[r]), a.hi[r]);
+                }
             }
-            q = make_par(th[0], th[1], th[2], th[3], th[4], q.delta);
+#pragma unroll
+            for (int r = 0; r < 5; ++r) sm[L::O_TH + r * 32 + lane] = th[r];
+        }
+        __syncthreads();
+        if (act) {
+            const float *x = sm + L::O_TH + lane;
+            q = make_par(x[0], x[32], x[64], x[96], x[128], q.delta);
         }
     }
-    if (act) {
+    if (w == 1 && act) {
 #pragma unroll
         for (int r = 0; r < 5; ++r) a.th[r][i] = th[r];
         if (bad) atomicOr(a.status, IDM_STATUS_NONFINITE);
     }
 }
 
-__global__ void __launch_bounds__(32) recon_fit_kernel(Args a)
+template <int D, int BLOCKS>
+__global__ void __launch_bounds__(32 * fit::W, BLOCKS) recon_fit_kernel(Args a)
 {
     extern __shared__ __align__(16) float sm[];
-    const int lane = threadIdx.x;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int i = blockIdx.x * 32 + lane;
     const bool act = i < a.N;
     const int Ki = horizon(a, i, act);
     const int Kw = __reduce_max_sync(FULL, (unsigned)Ki);
     const bool d4 = __all_sync(FULL, !act || a.th[5][i] == 4.0f);
     if (d4)
-        fit_warp<true>(a, i, act, Ki, Kw, sm, lane);
+        fit_block<true, D>(a, i, act, Ki, Kw, sm, lane, w);
     else
-        fit_warp<false>(a, i, act, Ki, Kw, sm, lane);
+        fit_block<false, D>(a, i, act, Ki, Kw, sm, lane, w);
 }
 
 // ---- preparation --------------------------------------------------------------
@@ -891,11 +1204,11 @@ int ensure_tape(idm_ctx *c, const idm_recon_t *r, rec::Args &a)
 }
 
 template <typename K>
-int launch_rec(idm_ctx *c, K kern, const rec::Args &a, cudaStream_t st)
+int launch_rec(idm_ctx *c, K kern, const rec::Args &a, cudaStream_t st, int warps = 1, int smem = rec::SMEM)
 {
     if (a.N == 0) return IDM_OK;
-    IDM_CK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, rec::SMEM));
-    kern<<<(a.N + 31) / 32, 32, rec::SMEM, st>>>(a);
+    IDM_CK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    kern<<<(a.N + 31) / 32, 32 * warps, smem, st>>>(a);
     IDM_CK(cudaGetLastError());
     return IDM_OK;
 }
@@ -997,12 +1310,14 @@ extern "C" int idm_recon_fit(idm_ctx_t *c, const idm_recon_t *r, idm_params_t *p
     if ((rc = ensure_status(c))) return rc;
     cudaStream_t st = (cudaStream_t)stream;
     rec::Args a = base_args(c, r, params, dp, dv);
-    if ((rc = build_obs_rows(c, r, a, st)) || (rc = ensure_tape(c, r, a))) return rc;
+    if ((rc = build_obs_rows(c, r, a, st))) return rc;
     const size_t rows = (size_t)r->k_max * r->ld, N = (size_t)r->n_traj;
+    if ((rc = ensure(c, c->rec_tape, sizeof(float) * 2 * rows, "fit tape"))) return rc;
+    a.tape_v = (float *)c->rec_tape.p;
+    a.tape_s = a.tape_v + rows;
     if ((rc = ensure(c, c->rec_mom, sizeof(float) * 4 * rows, "Adam moments of dp, dv"))) return rc;
     if ((rc = ensure(c, c->rec_thm, sizeof(float) * 10 * std::max<size_t>(N, 1), "Adam moments of the parameters")))
         return rc;
-    IDM_CK(cudaMemsetAsync(c->rec_mom.p, 0, sizeof(float) * 4 * rows, st));
     IDM_CK(cudaMemsetAsync(c->rec_thm.p, 0, sizeof(float) * 10 * std::max<size_t>(N, 1), st));
     a.mom = (float4 *)c->rec_mom.p;
     a.thm = (float *)c->rec_thm.p;
@@ -1016,7 +1331,13 @@ extern "C" int idm_recon_fit(idm_ctx_t *c, const idm_recon_t *r, idm_params_t *p
         a.hi[q] = box_hi[q];
     }
     if (loss_hist) IDM_CK(cudaMemsetAsync(loss_hist, 0, sizeof(double) * n_iter, st));
-    return launch_rec(c, rec::recon_fit_kernel, a, st);
+    // Two blocks per SM leave shared memory for copies two chunks ahead (97 KB),
+    // three for one (75 KB): measured per iteration on GB300, 6,101
+    // trajectories (191 blocks) 128 and 131 us, 21,750 (680 blocks) 280 and
+    // 261 us, 12,000 170 and 162 us.
+    if ((a.N + 31) / 32 <= 2 * c->n_sm)
+        return launch_rec(c, rec::recon_fit_kernel<2, 2>, a, st, rec::fit::W, rec::fit::Lay<2>::BYTES);
+    return launch_rec(c, rec::recon_fit_kernel<1, 3>, a, st, rec::fit::W, rec::fit::Lay<1>::BYTES);
 }
 
 extern "C" int idm_recon_metrics(idm_ctx_t *c, const idm_recon_t *r, const idm_params_t *params, const float *dp,
