@@ -93,6 +93,18 @@ unsigned long long *event_counters(idm_ctx *c)
     return reinterpret_cast<unsigned long long *>(static_cast<char *>(c->status.p) + STATUS_EVENTS_OFF);
 }
 
+// Segments of `cap` slots that N vehicles in L lanes (or L segments of a batch)
+// make, about: whole lanes of the mean length, at most 7/8 of the slots, and one
+// per lane chunk where the builder keeps all of them (launch_build_segments).
+static long long expected_segments(long long N, long long L, int cap)
+{
+    const long long full = (long long)cap * 7 / 8;
+    const long long lanes = std::max<long long>(1, cap / std::max<long long>(1, N / std::max<long long>(1, L)));
+    long long segs = std::max((N + full - 1) / full, (L + lanes - 1) / lanes);
+    if (N < 16 * L) segs = std::max<long long>(segs, idm::SEG_BUILD_CHUNKS);
+    return std::max<long long>(1, std::min<long long>(L, segs));
+}
+
 int pick_shape(idm_ctx *c, int max_lane, long long n_vehicles, int n_lanes, int *vpt, int *G)
 {
     int v = c->vpt_req, g = c->G_req;
@@ -103,6 +115,12 @@ int pick_shape(idm_ctx *c, int max_lane, long long n_vehicles, int n_lanes, int 
         g = 4;
         if (max_lane > 512) v = 8;
         if (max_lane > 1024) g = 8;
+        // up to two such segments per SM: 2 vehicles per thread x 8 warps (the
+        // same slots), two of those blocks per SM
+        if (max_lane <= 512 && expected_segments(n_vehicles, n_lanes, 512) <= 2LL * c->n_sm) {
+            v = 2;
+            g = 8;
+        }
         // a scene whose segments fit one wave of 2-vehicle warps (16 per SM)
         // is bound by the latency of each warp's step, not by throughput:
         // 2 vehicles per thread (the fewest instructions per step) and the
@@ -133,6 +151,8 @@ int pick_shape(idm_ctx *c, int max_lane, long long n_vehicles, int n_lanes, int 
     *G = g;
     return IDM_OK;
 }
+
+bool lanes_fit_one_wave(const idm_ctx *c, int n_lanes, int G) { return (long long)n_lanes * G <= 16LL * c->n_sm; }
 
 int check_scene(idm_ctx *c, const idm_scene_t *s)
 {
@@ -217,40 +237,49 @@ static int prepare(idm_ctx *c, const idm_scene_t *sc, const idm_params_t *pr, co
 
     CK(cudaMemsetAsync(c->ctl.p, 0, sizeof(int) * 3, st));
     CK(idm::launch_prep_gap(sc->lane_off, L, p_init, sc->length, N, (float *)c->g0.p, a.status, st));
-    CK(idm::launch_build_segments(sc->lane_off, L, nullptr, 0, 32 * P->vpt * G, N, (Seg *)c->seg.p,
-                                  (int *)c->ctl.p + CTL_NSEG, a.status, st));
+    CK(idm::launch_build_segments(sc->lane_off, L, 32 * P->vpt * G, N, lanes_fit_one_wave(c, L, G),
+                                  (Seg *)c->seg.p, (int *)c->ctl.p + CTL_NSEG, a.status, st));
     P->loss_per_seg = G;
     P->k_max = sim->K;
     return forward_grid(c, P, L);
 }
 
-void forward_shape(int vpt, int G, int *vpt_f, int *G_f)
+void forward_shape(int vpt, int G, long long segs, int n_sm, int *vpt_f, int *G_f)
 {
-    // the forward carries fewer live values per vehicle, so it prefers 8
-    // vehicles per thread (4 pairs of independent chains) for the same
-    // segment capacity, else 4
+    // The forward carries fewer live values per vehicle, so it runs 8 vehicles
+    // per thread (4 pairs of independent chains; 12 warps per SM) for the same
+    // segment capacity, else 4; or 2 when the segments then fit one wave of 16
+    // warps per SM (10 lanes of 100 over 100 steps: 33 -> 27 us; 4 per thread
+    // never won: 300 segments of 512 slots took 313 us for 300 steps against
+    // 261 with 8).
     const int cap = 32 * vpt * G;
-    if (cap % 256 == 0 && cap / 256 >= 1 && cap / 256 <= 8) {
-        *vpt_f = 8;
-        *G_f = cap / 256;
-    } else if (cap % 128 == 0 && cap / 128 >= 1 && cap / 128 <= 8) {
-        *vpt_f = 4;
-        *G_f = cap / 128;
-    } else {
-        *vpt_f = vpt;
-        *G_f = G;
-    }
+    auto fits = [&](int v) { return cap % (32 * v) == 0 && cap / (32 * v) >= 1 && cap / (32 * v) <= 8; };
+    int v = fits(8) ? 8 : (fits(4) ? 4 : vpt);
+    if (fits(2) && segs * (cap / 64) <= 16LL * n_sm) v = 2;
+    *vpt_f = v;
+    *G_f = v == vpt ? G : cap / (32 * v);
 }
 
 int forward_grid(idm_ctx *c, Prep *P, int L)
 {
-    forward_shape(P->vpt, P->G, &P->vpt_f, &P->G_f);
+    const long long segs = expected_segments(P->a.N_total, L, 32 * P->vpt * P->G);
+    forward_shape(P->vpt, P->G, segs, c->n_sm, &P->vpt_f, &P->G_f);
     const int G = P->G_f;
-    // 8 vehicles per thread: blocks of up to 12 warps (their register budget,
-    // one block per SM); otherwise the context's warps per block
-    P->wpb_f = P->vpt_f == 8 ? std::max(G, (12 / G) * G) : std::max(G, (c->wpb / G) * G);
-    // few segments: fewer per block, so that they spread over more SMs
-    P->wpb_f = std::min(P->wpb_f, G * std::max(1, (L + c->n_sm - 1) / c->n_sm));
+    if (P->vpt_f == 8) {
+        // 12 warps per SM (register budget).  Up to three segments per SM: a
+        // block each, so that they spread evenly; up to a wave: one block per
+        // SM; beyond: blocks of four warps, whose groups finish and refill
+        // independently (3,000 lanes of 60 over 300 steps, 375 segments: 230 us
+        // in 2-warp blocks, 300 in 4, 285 in 12; 1,400 x 180, 700 segments: 367,
+        // 299, 285; 5,000 x 100 over 1,000 steps, 1,000 segments: 1.32, 1.28,
+        // 1.55 ms)
+        const long long per_sm = 12 / G > 0 ? 12 / G : 1;
+        const int groups = segs <= 3LL * c->n_sm ? 1 : (segs <= per_sm * c->n_sm ? (int)per_sm : std::max(1, 4 / G));
+        P->wpb_f = G * groups;
+    } else {
+        // few segments: fewer per block, so that they spread over more SMs
+        P->wpb_f = std::min(std::max(G, (c->wpb / G) * G), G * (int)((segs + c->n_sm - 1) / c->n_sm));
+    }
     const int warps_needed = L * G;  // segments <= lanes
     const int blocks_needed = (warps_needed + P->wpb_f - 1) / P->wpb_f;
     int occ_f = idm::occupancy_blocks(P->vpt_f, G, false, false, false, false, P->wpb_f, 0);
@@ -309,7 +338,10 @@ int backward_grid(idm_ctx *c, Prep *P, bool dense, bool adam, bool want_delta, i
     const size_t per_group = idm::backward_smem_bytes(P->vpt, dense, T, G, G, pf);
     int groups = std::max(1, std::min(c->wpb / G, (int)(smem_max / per_group)));
     groups = std::max(1, std::min(groups, idm::backward_max_warps(P->vpt, G) / G));
-    groups = std::min(groups, std::max(1, (L + c->n_sm - 1) / c->n_sm));  // few segments: spread over the SMs
+    // few segments: spread over the SMs (in blocks of whole quarters of warps)
+    int spread = (int)((expected_segments(P->a.N_total, L, 32 * P->vpt * G) + c->n_sm - 1) / c->n_sm);
+    if (spread * G > 4) spread = ((spread * G + 3) / 4 * 4 + G - 1) / G;
+    groups = std::min(groups, spread);
     P->wpb_b = groups * G;
     size_t smem = per_group * groups;
     int occ_b = idm::occupancy_blocks(P->vpt, G, true, dense, adam, want_delta, P->wpb_b, smem, T < C);

@@ -82,8 +82,11 @@ unsigned long long *event_counters(idm_ctx *c);
 // for longer lanes), or for a scene that fits one wave of 2-vehicle warps
 // the latency shape 2 x G.
 int pick_shape(idm_ctx *c, int max_lane, long long n_vehicles, int n_lanes, int *vpt, int *G);
-// Forward shape for the segment capacity of the adjoint shape (vpt, G).
-void forward_shape(int vpt, int G, int *vpt_f, int *G_f);
+// Every lane as a segment of its own of G warps fits one wave of 16 warps per SM.
+bool lanes_fit_one_wave(const idm_ctx *c, int n_lanes, int G);
+// Forward shape for the segment capacity of the adjoint shape (vpt, G) and
+// about `segs` segments.
+void forward_shape(int vpt, int G, long long segs, int n_sm, int *vpt_f, int *G_f);
 // Parameter arrays: required unless the scene has no vehicles.
 int check_params(idm_ctx *c, const idm_params_t *p, bool all, long long n_vehicles);
 // Scene (lanes, lengths, max_lane) and simulation settings (K >= 1, finite

@@ -201,7 +201,8 @@ extern "C" int idm_loss_grad_noalloc(const idm_scene_t *sc, const idm_params_t *
     cudaError_t e = idm::launch_prep_gap(sc->lane_off, (int)L, p_init, sc->length, (int)N, (float *)(base + o_g0),
                                          status, st);
     if (e == cudaSuccess)
-        e = idm::launch_build_segments(sc->lane_off, (int)L, nullptr, 0, 32 * P.vpt * G, (int)N, (Seg *)(base + o_seg),
+        e = idm::launch_build_segments(sc->lane_off, (int)L, 32 * P.vpt * G, (int)N,
+                                       lanes_fit_one_wave(&c, (int)L, G), (Seg *)(base + o_seg),
                                        ctl + CTL_NSEG, status, st);
     if (e == cudaSuccess) {
         a.work = ctl + CTL_WORK_F;

@@ -52,89 +52,127 @@ cudaError_t launch_prep_gap(const int *lane_off, int n_lanes, const float *p_ini
 }
 
 // ---------------------------------------------------------------------------
-// Lane packing: each of 1024 threads packs a contiguous chunk of lanes
-// greedily into segments of at most `cap` vehicles (never across a scenario
-// boundary); a block scan places the chunks' segments.  A lane longer than
-// cap is skipped and flagged.
+// Lane packing: each thread packs a contiguous chunk of `per` lanes
+// greedily into segments of at most `cap` vehicles; a block scan places the
+// chunks' segments.  A lane longer than cap is skipped and flagged.
+//
+// A chunk's last segment is half empty on average, so a chunk holds about 32
+// segments' vehicles (with 1,024 chunks whatever the scene, 2,000 lanes of 100
+// made 1,000 segments of 2 lanes in 512 slots instead of 400 of 5, and the
+// simulation of such a scene took 1.4 to 2.3 times as long).  Scenes of short
+// lanes (under 16 vehicles), and those whose lanes fit one wave as segments of
+// their own (one_wave), keep 1,024 chunks.
+//
+// A thread that walked its chunk lane by lane would take ~25 us for 150 lanes.
+// With the offsets in shared memory (up to STAGED_LANES lanes) all threads first
+// find every lane's successor (the first lane that no longer fits a segment
+// starting there), and the walk jumps from segment to segment.
 // ---------------------------------------------------------------------------
 constexpr int BUILD_THREADS = SEG_BUILD_CHUNKS;
+constexpr int STAGED_LANES = 32768;
 
+__host__ __device__ inline size_t staged_bytes(int n_lanes) { return (size_t)(n_lanes + 1) * 6 + 16; }
+
+// One chunk lane by lane: more lanes than the staging holds, or lanes that are
+// malformed or longer than cap.
 template <bool EMIT>
-__device__ int pack_lanes(const int *lane_off, int l0, int l1, const int *scen_lane_off, int n_scen, int cap,
-                          int N, Seg *out, unsigned *status)
+__device__ int pack_lanes(const int *lane_off, int l0, int l1, int cap, int N, Seg *out, unsigned *status)
 {
-    int cnt = 0, fill = 0, seg_begin = 0, cur_scen = -1;
-    int s = 0;
-    if (scen_lane_off) {  // scenario of lane l0
-        int lo = 0, hi = n_scen - 1;
-        while (lo < hi) {
-            int mid = (lo + hi + 1) >> 1;
-            if (scen_lane_off[mid] <= l0) lo = mid; else hi = mid - 1;
-        }
-        s = lo;
-    }
+    int cnt = 0, fill = 0, seg_begin = 0;
     for (int l = l0; l < l1; ++l) {
-        if (scen_lane_off)
-            while (s + 1 < n_scen && scen_lane_off[s + 1] <= l) ++s;
-        int a = lane_off[l], e = lane_off[l + 1], n = e - a;
-        if (a < 0 || e > N || n < 0) {  // malformed: never read outside [0, N)
-            if (EMIT) atomicOr(status, IDM_STATUS_BAD_LANE_OFF);
-            if (fill > 0) {
-                if (EMIT) out[cnt] = Seg{seg_begin, fill, cur_scen < 0 ? 0 : cur_scen, 0};
-                ++cnt;
-                fill = 0;
-            }
-            continue;
-        }
-        if (n == 0) continue;
-        bool close = fill > 0 && (fill + n > cap || s != cur_scen);
-        if (n > cap) {
-            if (EMIT) atomicOr(status, IDM_STATUS_LANE_TOO_LONG);
-            close = fill > 0;
-        }
-        if (close) {
-            if (EMIT) out[cnt] = Seg{seg_begin, fill, cur_scen < 0 ? 0 : cur_scen, 0};
+        const int a = lane_off[l], e = lane_off[l + 1], n = e - a;
+        const bool bad = a < 0 || e > N || n < 0;  // malformed: never read outside [0, N)
+        const bool skip = bad || n > cap;
+        if (skip && EMIT) atomicOr(status, bad ? IDM_STATUS_BAD_LANE_OFF : IDM_STATUS_LANE_TOO_LONG);
+        if (fill > 0 && (skip || fill + n > cap)) {
+            if (EMIT) out[cnt] = Seg{seg_begin, fill, 0, 0};
             ++cnt;
             fill = 0;
         }
-        if (n > cap) continue;
-        if (fill == 0) { seg_begin = a; cur_scen = s; }
+        if (skip || n == 0) continue;
+        if (fill == 0) seg_begin = a;
         fill += n;
     }
     if (fill > 0) {
-        if (EMIT) out[cnt] = Seg{seg_begin, fill, cur_scen < 0 ? 0 : cur_scen, 0};
+        if (EMIT) out[cnt] = Seg{seg_begin, fill, 0, 0};
         ++cnt;
     }
     return cnt;
 }
 
 __global__ void __launch_bounds__(BUILD_THREADS)
-build_segments_kernel(const int *lane_off, int n_lanes, const int *scen_lane_off, int n_scen, int cap, int N,
-                      Seg *seg, int *n_seg, unsigned *status)
+build_segments_kernel(const int *lane_off, int n_lanes, int cap, int N, int per, bool staged, Seg *seg, int *n_seg,
+                      unsigned *status)
 {
+    extern __shared__ int off[];                                          // [n_lanes + 1] when staged
+    unsigned short *jump = reinterpret_cast<unsigned short *>(off + n_lanes + 1);  // lanes of the segment from a lane
     __shared__ int sc[BUILD_THREADS];
     const int t = threadIdx.x;
-    const int per = (n_lanes + BUILD_THREADS - 1) / BUILD_THREADS;
-    const int l0 = min(n_lanes, t * per), l1 = min(n_lanes, l0 + per);
-    int cnt = pack_lanes<false>(lane_off, l0, l1, scen_lane_off, n_scen, cap, N, nullptr, status);
+    const int l0 = (int)min((long long)n_lanes, (long long)t * per), l1 = min(n_lanes, l0 + per);
+    if (staged) {
+        for (int l = t; l <= n_lanes; l += BUILD_THREADS) off[l] = lane_off[l];
+        __syncthreads();
+        bool odd = false;
+        for (int l = t; l < n_lanes; l += BUILD_THREADS) {
+            const int a = off[l], e = off[l + 1];
+            odd |= a < 0 || e > N || e < a || e - a > cap;
+        }
+        staged = !__syncthreads_or(odd);
+    }
+    if (staged) {  // successors: two pointers over this thread's share of the lanes
+        const int share = (n_lanes + BUILD_THREADS - 1) / BUILD_THREADS;
+        const int s0 = min(n_lanes, t * share), s1 = min(n_lanes, s0 + share);
+        int m = s0;
+        for (int l = s0; l < s1; ++l) {
+            const int lim = off[l] + cap;
+            while (m < n_lanes && off[m + 1] <= lim) ++m;
+            jump[l] = (unsigned short)(m - l);
+        }
+        __syncthreads();
+    }
+    auto walk = [&](Seg *out) {  // this chunk by jumps
+        int cnt = 0;
+        for (int l = l0; l < l1;) {
+            const int m = min(l + (int)jump[l], l1), a = off[l], n = off[m] - a;
+            if (n > 0) {
+                if (out) out[cnt] = Seg{a, n, 0, 0};
+                ++cnt;
+            }
+            l = m;
+        }
+        return cnt;
+    };
+    const int cnt = staged ? walk(nullptr) : pack_lanes<false>(lane_off, l0, l1, cap, N, nullptr, status);
     sc[t] = cnt;
     __syncthreads();
-    for (int off = 1; off < BUILD_THREADS; off <<= 1) {  // inclusive Hillis-Steele scan
-        int v = t >= off ? sc[t - off] : 0;
+    for (int o = 1; o < BUILD_THREADS; o <<= 1) {  // inclusive Hillis-Steele scan
+        const int v = t >= o ? sc[t - o] : 0;
         __syncthreads();
         sc[t] += v;
         __syncthreads();
     }
-    int base = sc[t] - cnt;
-    pack_lanes<true>(lane_off, l0, l1, scen_lane_off, n_scen, cap, N, seg + base, status);
+    Seg *out = seg + (sc[t] - cnt);
+    if (staged)
+        walk(out);
+    else
+        pack_lanes<true>(lane_off, l0, l1, cap, N, out, status);
     if (t == BUILD_THREADS - 1) *n_seg = sc[t];
 }
 
-cudaError_t launch_build_segments(const int *lane_off, int n_lanes, const int *scen_lane_off, int n_scen,
-                                  int cap, int N, Seg *seg, int *n_seg, unsigned *status, cudaStream_t st)
+cudaError_t launch_build_segments(const int *lane_off, int n_lanes, int cap, int N, bool one_wave, Seg *seg, int *n_seg,
+                                  unsigned *status, cudaStream_t st)
 {
-    build_segments_kernel<<<1, BUILD_THREADS, 0, st>>>(lane_off, n_lanes, scen_lane_off, n_scen, cap, N, seg,
-                                                       n_seg, status);
+    // 32 segments of as many whole lanes of the mean length as fit
+    const long long mean = N > 0 ? ((long long)N + n_lanes - 1) / n_lanes : 1;
+    const long long full = 32 * (mean < cap ? cap / mean : 1), least = ((long long)n_lanes + BUILD_THREADS - 1) / BUILD_THREADS;
+    const bool short_lanes = (long long)N < 16LL * n_lanes;
+    const int per = (int)(one_wave || short_lanes || full < least ? least : full);  // lanes per chunk
+    const bool staged = n_lanes <= STAGED_LANES;
+    const size_t smem = staged ? staged_bytes(n_lanes) : 0;
+    cudaError_t e = cudaFuncSetAttribute(build_segments_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)staged_bytes(STAGED_LANES));
+    if (e != cudaSuccess) return e;
+    build_segments_kernel<<<1, BUILD_THREADS, smem, st>>>(lane_off, n_lanes, cap, N, per, staged, seg, n_seg, status);
     return cudaGetLastError();
 }
 
