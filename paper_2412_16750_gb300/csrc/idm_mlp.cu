@@ -42,6 +42,34 @@ constexpr int OFF_W1 = 0, OFF_B1 = OFF_W1 + HID * IN, OFF_W2 = OFF_B1 + HID, OFF
               OFF_B4 = OFF_W4 + OUT * HID, NPARAM = OFF_B4 + OUT;
 static_assert(NPARAM == IDM_MLP_N_PARAMS, "parameter count");
 
+// Programmatic dependent launch: a kernel launched with the attribute may start
+// while its predecessor in the stream still runs; pdl_wait returns when that has
+// completed (at once without the attribute) and lets the successor start in
+// turn.  Everything a kernel does before it (barriers, tensor memory, weights
+// that no kernel of the chain writes) overlaps the predecessor.  Since each
+// kernel of the chain waits before it triggers, a completed predecessor means
+// all earlier kernels have completed too.
+__device__ __forceinline__ void pdl_wait()
+{
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+template <typename K, typename... A>
+cudaError_t launch_pdl(K kern, dim3 grid, int threads, size_t smem, cudaStream_t st, bool dependent, const A &...args)
+{
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = &at;
+    cfg.numAttrs = dependent ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kern, args...);
+}
+
 enum Mode { GELU_FWD = 0, OUT_TRAIN = 1, OUT_INFER = 2, DGELU = 3, F32_PART = 4 };
 
 struct GemmArgs {
@@ -302,10 +330,10 @@ __device__ __forceinline__ void epilogue_row(const GemmArgs &g, int r, uint32_t 
     }
 }
 
+// One CTA's tile (bx, by) of K split bz.
 template <int MODE>
-__global__ void __launch_bounds__(tc::NTHREADS) mlp_gemm_kernel(const GemmArgs g)
+__device__ __forceinline__ void gemm_tile(const GemmArgs &g, int bx, int by, int bz, uint8_t *smem, bool dependent)
 {
-    extern __shared__ __align__(128) uint8_t smem[];
     const int BN = g.BN;
     const uint32_t ncols = tc::tmem_cols_for(BN);
     uint8_t *ctl = smem + 2 * tc::A_STAGE_BYTES + 2 * tc::b_stage_bytes(BN);
@@ -322,28 +350,36 @@ __global__ void __launch_bounds__(tc::NTHREADS) mlp_gemm_kernel(const GemmArgs g
     __syncthreads();
     tc::fence_after_sync();
     const uint32_t tmem = *tmem_slot;
+    if (dependent) pdl_wait();
 
     tc::TileArgs t;
     t.A = g.A;
     t.B = g.B;
     t.K = g.K;
     t.M_valid = g.M_valid;
-    t.m0 = blockIdx.x * tc::BM;
-    t.n0 = blockIdx.y * BN;
+    t.m0 = bx * tc::BM;
+    t.n0 = by * BN;
     t.BN = BN;
-    t.kb = blockIdx.z * g.k_chunk;
+    t.kb = bz * g.k_chunk;
     t.ke = min(g.K, t.kb + g.k_chunk);
     bool empty = false;
     const bool ok = tc::mainloop(t, smem, tmem, g.status, &empty, g.wait_iters);
     if (ok)
-        epilogue_row<MODE>(g, t.m0 + threadIdx.x, tmem + ((uint32_t)(warp * 32) << 16), t.n0, 0, t.BN, empty, blockIdx.z,
-                           blockIdx.x * 4 + warp, g.bias);
+        epilogue_row<MODE>(g, t.m0 + threadIdx.x, tmem + ((uint32_t)(warp * 32) << 16), t.n0, 0, t.BN, empty, bz,
+                           bx * 4 + warp, g.bias);
     tc::fence_before_sync();
     __syncthreads();
     if (warp == 0) {
         tc::fence_after_sync();
         tc::tmem_dealloc(tmem, ncols);
     }
+}
+
+template <int MODE>
+__global__ void __launch_bounds__(tc::NTHREADS) mlp_gemm_kernel(const GemmArgs g)
+{
+    extern __shared__ __align__(128) uint8_t smem[];
+    gemm_tile<MODE>(g, blockIdx.x, blockIdx.y, blockIdx.z, smem, false);
 }
 
 // Host launch of one GEMM; grid = (ceil(M/128), N/BN, splits).
@@ -356,6 +392,23 @@ cudaError_t gemm(const GemmArgs &g, int M_tiles_rows, int splits, cudaStream_t s
     dim3 grid((M_tiles_rows + tc::BM - 1) / tc::BM, g.N / g.BN, splits);
     mlp_gemm_kernel<MODE><<<grid, tc::NTHREADS, smem, st>>>(g);
     return cudaGetLastError();
+}
+
+// The weight gradients of all layers in one launch: block x is one 128 x BN
+// tile of one product, block y one K split.  (One launch per layer: 13 us each
+// at a batch of 8,192, almost all of it ramp and the latency of four K tiles;
+// together 4 CTAs per SM hide each other's.)
+struct WgradArgs {
+    GemmArgs g[4];
+    int tiles[5];  // first tile of product l, and their sum
+};
+__global__ void __launch_bounds__(tc::NTHREADS) mlp_wgrad_kernel(const __grid_constant__ WgradArgs w)
+{
+    extern __shared__ __align__(128) uint8_t smem[];
+    int l = 0;
+    while ((int)blockIdx.x >= w.tiles[l + 1]) ++l;
+    const int tile = blockIdx.x - w.tiles[l];
+    gemm_tile<F32_PART>(w.g[l], tile & 1, tile >> 1, blockIdx.y, smem, true);
 }
 
 // ---------------------------------------------------------------------------
@@ -445,6 +498,7 @@ __global__ void __launch_bounds__(ws::NTHREADS, 1)
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         __syncwarp();
         if (lane == 0) tc::mbar_arrive(wbar);
+        pdl_wait();  // A and the epilogue's inputs are the predecessors' outputs
         int q = 0;
         bool ok = true;
         for (int tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x) {
@@ -590,7 +644,7 @@ cudaError_t a_tensor_map(const GemmArgs &g, CUtensorMap *tm)
 // Launch of the persistent GEMM: CTAs keep column slices of nsplit equal
 // parts of the weights; each walks row tiles (grid x) of its slice (grid y).
 template <int MODE>
-cudaError_t gemm_ws(const GemmArgs &g0, int n_sm, int nsplit, cudaStream_t st)
+cudaError_t gemm_ws(const GemmArgs &g0, int n_sm, int nsplit, bool dependent, cudaStream_t st)
 {
     GemmArgs g = g0;
     g.BN = g.N / nsplit;
@@ -612,23 +666,24 @@ cudaError_t gemm_ws(const GemmArgs &g0, int n_sm, int nsplit, cudaStream_t st)
     const int grid = std::max(1, std::min(ntiles, (n_sm * occ + nsplit - 1) / nsplit));
     CUtensorMap tmA;
     if ((e = a_tensor_map(g, &tmA)) != cudaSuccess) return e;
-    mlp_gemm_ws_kernel<MODE><<<dim3(grid, nsplit), ws::NTHREADS, smem, st>>>(g, tmA);
-    return cudaGetLastError();
+    return launch_pdl(mlp_gemm_ws_kernel<MODE>, dim3(grid, nsplit), ws::NTHREADS, smem, st, dependent, g, tmA);
 }
 
 // Batch-sized product: the persistent kernel when there are enough row tiles
 // to keep every SM busy for several tiles (it loads the whole weight matrix
 // once per CTA and overlaps each tile's epilogue with the next tile's
 // products), else one CTA per 128 x BN tile.
+// dependent: the predecessor in the stream is a kernel of this network's chain
+// that does not write the weights.
 template <int MODE>
-cudaError_t gemm_batch(const GemmArgs &g, int n_sm, cudaStream_t st)
+cudaError_t gemm_batch(const GemmArgs &g, int n_sm, bool dependent, cudaStream_t st)
 {
     const int ntiles = (g.M_rows + tc::BM - 1) / tc::BM;
     // few row tiles: split the columns so that more SMs work (each CTA then
     // keeps a narrower weight slice)
     int nsplit = 1;
     while (ntiles * nsplit < n_sm && g.N / (2 * nsplit) >= 64 && (g.N / (2 * nsplit)) % 16 == 0) nsplit *= 2;
-    return gemm_ws<MODE>(g, n_sm, nsplit, st);
+    return gemm_ws<MODE>(g, n_sm, nsplit, dependent, st);
 }
 
 // ---------------------------------------------------------------------------
@@ -666,43 +721,65 @@ __device__ __forceinline__ float obs_at(const FeatArgs &f, int i, int j)
     return j == 0 ? f.p_init[i] : f.targets[(size_t)(j - 1) * f.N + i];
 }
 
-__global__ void __launch_bounds__(128) features_kernel(const FeatArgs f)
+// One thread per row; the block's rows are staged in shared memory (41 words a
+// row, so that the threads' words fall in different banks) and leave as one
+// contiguous run of words.  HBM-bound in principle (80 B in, 160 B out per
+// row); with each thread writing its own 160-byte row from an array in local
+// memory 200,000 rows took 53 us.
+constexpr int FEAT_THREADS = 128, FEAT_WORDS = IN / 2;
+
+__global__ void __launch_bounds__(FEAT_THREADS) features_kernel(const FeatArgs f)
 {
-    const int r = blockIdx.x * blockDim.x + threadIdx.x;
-    if (r >= f.n_rows) return;
-    const int i = f.perm ? f.perm[r] : r;
-    if (i < 0 || i >= f.N) return;
-    const bool head = is_lane_head(f.lane_off, f.n_lanes, i);
-    const float inv_2sdt = 1.0f / (2.0f * (float)f.obs_stride * f.dt);
-    const float y0 = f.p_init[i];
-    float feat[4 * PREFIX];
-    for (int who = 0; who < 2; ++who) {
-        const int k = who == 0 ? i : i - 1;
-        float *x = feat + 2 * PREFIX * who, *v = x + PREFIX;
-        if (who == 1 && head) {
-            for (int j = 0; j < PREFIX; ++j) {
-                x[j] = feat[j] + 2.0f;
-                v[j] = feat[PREFIX + j];
+    __shared__ uint32_t stage[FEAT_THREADS][FEAT_WORDS + 1];
+    __shared__ bool live[FEAT_THREADS];
+    const int r = blockIdx.x * FEAT_THREADS + threadIdx.x;
+    const int i = r < f.n_rows ? (f.perm ? f.perm[r] : r) : -1;
+    const bool ok = i >= 0 && i < f.N;
+    live[threadIdx.x] = ok;
+    if (ok) {
+        const bool head = is_lane_head(f.lane_off, f.n_lanes, i);
+        const float inv_2sdt = 1.0f / (2.0f * (float)f.obs_stride * f.dt);
+        const float y0 = f.p_init[i];
+        uint32_t *out = stage[threadIdx.x];
+        auto pack = [](float a, float b) {
+            const __nv_bfloat162 v = __floats2bfloat162_rn(a, b);
+            return *reinterpret_cast<const uint32_t *>(&v);
+        };
+        // vehicle k's positions and speeds into words [w, w + 10) and [w + 10,
+        // w + 20); a head's leader (the vehicle itself, 200 m ahead) into the
+        // words of the leader as well
+        auto series = [&](int k, int w, bool virt) {
+            float prev = obs_at(f, k, 0), cur = obs_at(f, k, 1);
+            float xa = (prev - y0) / 100.0f, va = f.v_init[k] / 30.0f;
+#pragma unroll
+            for (int j = 1; j < PREFIX; ++j) {
+                const float next = obs_at(f, k, j + 1);
+                const float x = (cur - y0) / 100.0f, v = (next - prev) * inv_2sdt / 30.0f;
+                if (j & 1) {
+                    const uint32_t vw = pack(va, v);
+                    out[w + j / 2] = pack(xa, x);
+                    out[w + PREFIX / 2 + j / 2] = vw;
+                    if (virt) {
+                        out[w + PREFIX + j / 2] = pack(xa + 2.0f, x + 2.0f);
+                        out[w + 3 * PREFIX / 2 + j / 2] = vw;
+                    }
+                }
+                xa = x;
+                va = v;
+                prev = cur;
+                cur = next;
             }
-            break;
-        }
-        float prev = obs_at(f, k, 0), cur = obs_at(f, k, 1);
-        x[0] = (prev - y0) / 100.0f;
-        v[0] = f.v_init[k] / 30.0f;
-        for (int j = 1; j < PREFIX; ++j) {
-            const float next = obs_at(f, k, j + 1);
-            x[j] = (cur - y0) / 100.0f;
-            v[j] = (next - prev) * inv_2sdt / 30.0f;
-            prev = cur;
-            cur = next;
-        }
+        };
+        series(i, 0, head);
+        if (!head) series(i - 1, PREFIX, false);
+        if (f.labels)
+            for (int q = 0; q < OUT; ++q) f.labels[(size_t)r * OUT + q] = (f.th[q][i] - f.lo[q]) / (f.hi[q] - f.lo[q]);
     }
-    __align__(16) bf16 row[4 * PREFIX];
-    for (int q = 0; q < 4 * PREFIX; ++q) row[q] = __float2bfloat16_rn(feat[q]);
-    uint4 *dst = reinterpret_cast<uint4 *>(f.X + (size_t)r * IN);
-    for (int q = 0; q < IN / 8; ++q) dst[q] = reinterpret_cast<const uint4 *>(row)[q];
-    if (f.labels) {
-        for (int q = 0; q < OUT; ++q) f.labels[(size_t)r * OUT + q] = (f.th[q][i] - f.lo[q]) / (f.hi[q] - f.lo[q]);
+    __syncthreads();
+    uint32_t *dst = reinterpret_cast<uint32_t *>(f.X) + (size_t)blockIdx.x * FEAT_THREADS * FEAT_WORDS;
+    for (int k = threadIdx.x; k < FEAT_THREADS * FEAT_WORDS; k += FEAT_THREADS) {
+        const int row = k / FEAT_WORDS;
+        if (live[row]) dst[k] = stage[row][k - row * FEAT_WORDS];
     }
 }
 
@@ -710,36 +787,75 @@ __global__ void __launch_bounds__(128) features_kernel(const FeatArgs f)
 // Small kernels: transpose of the input batch, column sums (bias
 // gradients), the parameter update, the loss reduction.
 // ---------------------------------------------------------------------------
-// out[c][r] = in[r][c] for r < rows_valid, 0 for rows_valid <= r < rows_pad.
-__global__ void transpose_kernel(const bf16 *in, int rows_valid, int rows_pad, int cols, bf16 *out)
-{
-    __shared__ bf16 tile[32][33];
-    const int r0 = blockIdx.x * 32, c0 = blockIdx.y * 32;
-    for (int y = threadIdx.y; y < 32; y += blockDim.y) {
-        const int r = r0 + y, c = c0 + threadIdx.x;
-        tile[y][threadIdx.x] = (r < rows_valid && c < cols) ? in[(size_t)r * cols + c] : __float2bfloat16_rn(0.0f);
-    }
-    __syncthreads();
-    for (int y = threadIdx.y; y < 32; y += blockDim.y) {
-        const int c = c0 + y, r = r0 + threadIdx.x;
-        if (c < cols && r < rows_pad) out[(size_t)c * rows_pad + r] = tile[threadIdx.x][y];
-    }
-}
+// One launch for the small work between the backward products and the weight
+// gradients, by block index: the transpose of the input batch (out[c][r] =
+// in[r][c] for r < rows_valid, 0 for rows_valid <= r < rows_pad; 32 x 32 tiles),
+// the bias gradients (row sums of the transposed dO and dZ, FP32, fixed order)
+// and the loss (FP64 sum of the output layer's partials).
+struct AuxArgs {
+    const bf16 *X;            // [rows_valid][IN]
+    int rows_valid, rows_pad;
+    bf16 *XT;                 // [IN][rows_pad]
+    const bf16 *dOT, *dZT[3]; // [OUTP][rows_pad], [HID][rows_pad]
+    float *db;                // [3 HID + OUTP]: db1, db2, db3, db4
+    const double *part;       // [n_part]
+    int n_part;
+    double *loss;
+    unsigned *status;
+};
+constexpr int AUX_THREADS = 256;
+__host__ __device__ inline int aux_tiles(int rows_pad) { return rows_pad / 32 * ((IN + 31) / 32); }
+__host__ __device__ inline int aux_blocks(int rows_pad) { return 1 + 3 * HID + OUTP + aux_tiles(rows_pad); }
 
-// out[row] = sum_{c < n} in[row][c] (FP32, fixed order).
-__global__ void __launch_bounds__(256) colsum_kernel(const bf16 *in, int ld, int n, float *out)
+__global__ void __launch_bounds__(AUX_THREADS) aux_kernel(const AuxArgs x)
 {
-    __shared__ float sh[256];
-    const bf16 *p = in + (size_t)blockIdx.x * ld;
-    float s = 0.0f;
-    for (int c = threadIdx.x; c < n; c += 256) s += __bfloat162float(p[c]);
-    sh[threadIdx.x] = s;
-    __syncthreads();
-    for (int o = 128; o > 0; o >>= 1) {
-        if ((int)threadIdx.x < o) sh[threadIdx.x] += sh[threadIdx.x + o];
+    pdl_wait();
+    __shared__ double sh[AUX_THREADS];
+    const int t = threadIdx.x;
+    int b = blockIdx.x;
+    if (b == 0) {
+        double s = 0.0;
+        for (int i = t; i < x.n_part; i += AUX_THREADS) s += x.part[i];
+        sh[t] = s;
         __syncthreads();
+        for (int o = AUX_THREADS / 2; o > 0; o >>= 1) {
+            if (t < o) sh[t] += sh[t + o];
+            __syncthreads();
+        }
+        if (t == 0) {
+            if (!isfinite(sh[0])) atomicOr(x.status, IDM_STATUS_NONFINITE);
+            if (x.loss) *x.loss = sh[0];
+        }
+        return;
     }
-    if (threadIdx.x == 0) out[blockIdx.x] = sh[0];
+    b -= 1;
+    if (b < 3 * HID + OUTP) {
+        float *sf = reinterpret_cast<float *>(sh);
+        const bf16 *p = (b < 3 * HID ? x.dZT[b / HID] + (size_t)(b % HID) * x.rows_pad
+                                     : x.dOT + (size_t)(b - 3 * HID) * x.rows_pad);
+        float s = 0.0f;
+        for (int c = t; c < x.rows_pad; c += AUX_THREADS) s += __bfloat162float(p[c]);
+        sf[t] = s;
+        __syncthreads();
+        for (int o = AUX_THREADS / 2; o > 0; o >>= 1) {
+            if (t < o) sf[t] += sf[t + o];
+            __syncthreads();
+        }
+        if (t == 0) x.db[b] = sf[0];
+        return;
+    }
+    b -= 3 * HID + OUTP;
+    __shared__ bf16 tile[32][33];
+    const int cols = (IN + 31) / 32, r0 = b / cols * 32, c0 = b % cols * 32, tx = t & 31;
+    for (int y = t >> 5; y < 32; y += AUX_THREADS / 32) {
+        const int r = r0 + y, c = c0 + tx;
+        tile[y][tx] = (r < x.rows_valid && c < IN) ? x.X[(size_t)r * IN + c] : __float2bfloat16_rn(0.0f);
+    }
+    __syncthreads();
+    for (int y = t >> 5; y < 32; y += AUX_THREADS / 32) {
+        const int c = c0 + y, r = r0 + tx;
+        if (c < IN) x.XT[(size_t)c * x.rows_pad + r] = tile[tx][y];
+    }
 }
 
 struct UpdArgs {
@@ -757,12 +873,21 @@ struct UpdArgs {
 __device__ __forceinline__ float sum_parts(const float *P, int S, size_t stride, size_t idx)
 {
     float s = 0.0f;
-    for (int q = 0; q < S; ++q) s += P[q * stride + idx];
+    int q = 0;
+    for (; q + 8 <= S; q += 8) {  // eight loads in flight
+        float v[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) v[j] = P[(q + j) * stride + idx];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) s += v[j];
+    }
+    for (; q < S; ++q) s += P[q * stride + idx];
     return s;
 }
 
 __global__ void __launch_bounds__(256) update_kernel(const UpdArgs u)
 {
+    pdl_wait();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= NPARAM) return;
     int layer, o, j, in_dim, outp;
@@ -805,23 +930,6 @@ __global__ void __launch_bounds__(256) update_kernel(const UpdArgs u)
     }
 }
 
-__global__ void loss_sum_kernel(const double *part, int n, double *out, unsigned *status)
-{
-    __shared__ double sh[256];
-    double s = 0.0;
-    for (int i = threadIdx.x; i < n; i += blockDim.x) s += part[i];
-    sh[threadIdx.x] = s;
-    __syncthreads();
-    for (int o = blockDim.x / 2; o > 0; o >>= 1) {
-        if ((int)threadIdx.x < o) sh[threadIdx.x] += sh[threadIdx.x + o];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) {
-        if (!isfinite(sh[0])) atomicOr(status, IDM_STATUS_NONFINITE);
-        if (out) *out = sh[0];
-    }
-}
-
 }  // namespace mlp
 }  // namespace idm
 
@@ -835,7 +943,7 @@ struct idm_mlp {
     void *arena = nullptr;
     float *w = nullptr, *m = nullptr, *v = nullptr;
     bf16 *Wb[4] = {}, *Wt[4] = {};
-    bf16 *XT = nullptr, *H[3] = {}, *HT[3] = {}, *dO = nullptr, *dOT = nullptr, *dZ[2] = {}, *dZT[2] = {};
+    bf16 *XT = nullptr, *H[3] = {}, *HT[3] = {}, *dO = nullptr, *dOT = nullptr, *dZ[2] = {}, *dZT[3] = {};
     float *Z[3] = {};
     float *P[4] = {};
     float *db = nullptr;
@@ -872,15 +980,16 @@ int mfail(idm_mlp *n, int code, const char *fmt, ...)
 
 int round128(int x) { return (x + 127) / 128 * 128; }
 
-// Split-K plan of a weight-gradient GEMM: K = Bp rows of the batch.
-void wgrad_plan(int n_sm, int Bp, int m_tiles, int n_tiles, int *splits, int *k_chunk)
+// Weight-gradient products (rows of the transposed left operand HID; columns
+// of a tile) and their split of K = Bp rows of the batch: four CTAs per SM
+// over the WG_TILES tiles, at least 256 rows each.
+constexpr int WG_BN[4] = {IN, 64, 64, OUTP}, WG_N[4] = {IN, HID, HID, OUTP};
+constexpr int WG_TILES = HID / 128 * (IN / WG_BN[0] + HID / WG_BN[1] + HID / WG_BN[2] + OUTP / WG_BN[3]);
+void wgrad_plan(int n_sm, int Bp, int *splits, int *k_chunk)
 {
-    int S = std::max(1, 2 * n_sm / std::max(1, m_tiles * n_tiles));
-    S = std::min(S, std::max(1, Bp / 256));
-    int kc = (Bp + S - 1) / S;
-    kc = (kc + 63) / 64 * 64;
-    *k_chunk = kc;
-    *splits = (Bp + kc - 1) / kc;
+    const int S = std::max(1, std::min(4 * n_sm / WG_TILES, Bp / 256));
+    *k_chunk = ((Bp + S - 1) / S + 63) / 64 * 64;
+    *splits = (Bp + *k_chunk - 1) / *k_chunk;
 }
 
 GemmArgs base_args(idm_mlp *n)
@@ -916,7 +1025,7 @@ int hidden_forward(idm_mlp *n, const bf16 *X, int B, int Bp, bool store_train, c
         g.H = dst;
         g.HT = store_train ? n->HT[l] : nullptr;
         g.ldt = Bp;
-        MCK(gemm_batch<GELU_FWD>(g, n->n_sm, st));
+        MCK(gemm_batch<GELU_FWD>(g, n->n_sm, l > 0, st));
     }
     return IDM_OK;
 }
@@ -927,12 +1036,6 @@ int fwd_bwd(idm_mlp *n, const bf16 *X, const float *labels, int B, double *loss_
 {
     const int Bp = round128(B);
     int rc;
-    // X^T for dW1
-    {
-        dim3 grid(Bp / 32, (IN + 31) / 32), block(32, 8);
-        idm::mlp::transpose_kernel<<<grid, block, 0, st>>>(X, B, Bp, IN, n->XT);
-        MCK(cudaGetLastError());
-    }
     if ((rc = hidden_forward(n, X, B, Bp, true, st))) return rc;
     {  // output layer + loss + dO
         GemmArgs g = base_args(n);
@@ -951,74 +1054,64 @@ int fwd_bwd(idm_mlp *n, const bf16 *X, const float *labels, int B, double *loss_
         g.label = labels;
         g.loss_part = n->loss_part;
         g.scale = 1.0f / (5.0f * (float)B);
-        MCK(gemm_batch<OUT_TRAIN>(g, n->n_sm, st));
-        idm::mlp::loss_sum_kernel<<<1, 256, 0, st>>>(n->loss_part, Bp / 128 * 4, loss_out ? loss_out : n->loss_tmp,
-                                                      n->status);
-        MCK(cudaGetLastError());
+        MCK(gemm_batch<OUT_TRAIN>(g, n->n_sm, true, st));
     }
-    // dW4^T = H3^T . dO  (M = 256 hidden units, N = 16, K = Bp)
-    int S, kc;
-    wgrad_plan(n->n_sm, Bp, 2, 1, &S, &kc);
-    {
+    // hidden layers, top down: dZ_l = (dZ_{l+1} W_{l+1}) * gelu'(Z_l)
+    for (int l = 2; l >= 0; --l) {
         GemmArgs g = base_args(n);
-        g.A = n->HT[2];
-        g.B = n->dOT;
+        g.A = l == 2 ? n->dO : n->dZ[(l + 1) & 1];
+        g.B = n->Wt[l + 1];  // W_{l+1}^T [256][width]
+        g.M_valid = Bp;
+        g.M_rows = Bp;
+        g.N = HID;
+        g.K = l == 2 ? OUTP : HID;
+        g.BN = 128;
+        g.k_chunk = g.K;
+        g.Z = n->Z[l];
+        g.H = l > 0 ? n->dZ[l & 1] : nullptr;
+        g.HT = n->dZT[l];
+        g.ldt = Bp;
+        MCK(gemm_batch<DGELU>(g, n->n_sm, true, st));
+    }
+    {  // X^T for dW1, the bias gradients and the loss
+        AuxArgs x;
+        x.X = X;
+        x.rows_valid = B;
+        x.rows_pad = Bp;
+        x.XT = n->XT;
+        x.dOT = n->dOT;
+        for (int l = 0; l < 3; ++l) x.dZT[l] = n->dZT[l];
+        x.db = n->db;
+        x.part = n->loss_part;
+        x.n_part = Bp / 128 * 4;
+        x.loss = loss_out ? loss_out : n->loss_tmp;
+        x.status = n->status;
+        MCK(launch_pdl(idm::mlp::aux_kernel, dim3(aux_blocks(Bp)), AUX_THREADS, 0, st, true, x));
+    }
+    // dW_l = dZ_l^T . H_{l-1} (M = 256, N = fan-in, K = Bp), dW4^T = H3^T . dO
+    int S, kc, bn = 0;
+    wgrad_plan(n->n_sm, Bp, &S, &kc);
+    WgradArgs w;
+    w.tiles[0] = 0;
+    for (int l = 0; l < 4; ++l) {
+        GemmArgs &g = w.g[l];
+        g = base_args(n);
+        g.A = l < 3 ? n->dZT[l] : n->HT[2];
+        g.B = l == 0 ? n->XT : (l < 3 ? n->HT[l - 1] : n->dOT);
         g.M_valid = HID;
         g.M_rows = HID;
-        g.N = OUTP;
+        g.N = WG_N[l];
         g.K = Bp;
-        g.BN = OUTP;
+        g.BN = WG_BN[l];
         g.k_chunk = kc;
-        g.Cf = n->P[3];
-        MCK(gemm<F32_PART>(g, HID, S, st));
-        u->S[3] = S;
+        g.Cf = n->P[l];
+        w.tiles[l + 1] = w.tiles[l] + HID / 128 * (g.N / g.BN);
+        bn = std::max(bn, g.BN);
+        u->S[l] = S;
     }
-    idm::mlp::colsum_kernel<<<OUTP, 256, 0, st>>>(n->dOT, Bp, Bp, n->db + 3 * HID);
-    MCK(cudaGetLastError());
-    // hidden layers, top down: dZ_l = (dZ_{l+1} W_{l+1}) * gelu'(Z_l)
-    const bf16 *up = n->dO;  // dZ_{l+1} as [Bp][width]
-    int up_width = OUTP;
-    for (int l = 2; l >= 0; --l) {
-        const int buf = l & 1;
-        {
-            GemmArgs g = base_args(n);
-            g.A = up;
-            g.B = n->Wt[l + 1];  // W_{l+1}^T [256][width]
-            g.M_valid = Bp;
-            g.M_rows = Bp;
-            g.N = HID;
-            g.K = up_width;
-            g.BN = 128;
-            g.k_chunk = up_width;
-            g.Z = n->Z[l];
-            g.H = l > 0 ? n->dZ[buf] : nullptr;
-            g.HT = n->dZT[buf];
-            g.ldt = Bp;
-            MCK(gemm_batch<DGELU>(g, n->n_sm, st));
-        }
-        // dW_l = dZ_l^T . H_{l-1}  (M = 256, N = fan-in, K = Bp)
-        {
-            const int fan_in = l == 0 ? IN : HID;
-            const int bn = l == 0 ? IN : 64;
-            wgrad_plan(n->n_sm, Bp, 2, fan_in / bn, &S, &kc);
-            GemmArgs g = base_args(n);
-            g.A = n->dZT[buf];
-            g.B = l == 0 ? n->XT : n->HT[l - 1];
-            g.M_valid = HID;
-            g.M_rows = HID;
-            g.N = fan_in;
-            g.K = Bp;
-            g.BN = bn;
-            g.k_chunk = kc;
-            g.Cf = n->P[l];
-            MCK(gemm<F32_PART>(g, HID, S, st));
-            u->S[l] = S;
-        }
-        idm::mlp::colsum_kernel<<<HID, 256, 0, st>>>(n->dZT[buf], Bp, Bp, n->db + l * HID);
-        MCK(cudaGetLastError());
-        up = n->dZ[buf];
-        up_width = HID;
-    }
+    const int smem = tc::smem_bytes(bn);
+    MCK(cudaFuncSetAttribute(idm::mlp::mlp_wgrad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    MCK(launch_pdl(idm::mlp::mlp_wgrad_kernel, dim3(w.tiles[4], S), tc::NTHREADS, smem, st, true, w));
     return IDM_OK;
 }
 
@@ -1070,8 +1163,8 @@ UpdArgs upd_base(idm_mlp *n)
 
 cudaError_t launch_update(const UpdArgs &u, cudaStream_t st)
 {
-    idm::mlp::update_kernel<<<(NPARAM + 255) / 256, 256, 0, st>>>(u);
-    return cudaGetLastError();
+    // (mode 0 follows copies, not a kernel of the chain)
+    return launch_pdl(idm::mlp::update_kernel, dim3((NPARAM + 255) / 256), 256, 0, st, u.mode != 0, u);
 }
 
 int check_batch(idm_mlp *n, const void *X, int B)
@@ -1140,13 +1233,9 @@ int idm_mlp_create(idm_mlp_t **out, int32_t max_batch)
     n->max_batch = max_batch;
     const int Bp = round128(max_batch);
     n->bp_cap = Bp;
-    // largest split count any weight-gradient GEMM uses at this batch size
-    int S = 1;
-    for (int tiles : {1, 4}) {
-        int s_, k_;
-        wgrad_plan(n->n_sm, Bp, 2, tiles, &s_, &k_);
-        S = std::max(S, s_);
-    }
+    int S, k_chunk;  // no smaller batch has more splits
+    wgrad_plan(n->n_sm, Bp, &S, &k_chunk);
+    S = std::max(S, std::max(1, std::min(4 * n->n_sm / WG_TILES, Bp / 256)));
     n->S_cap = S;
     // carve one arena
     size_t off = 0;
@@ -1166,17 +1255,15 @@ int idm_mlp_create(idm_mlp_t **out, int32_t max_batch)
     o_Wt[2] = take(2 * (size_t)HID * HID);
     o_Wt[3] = take(2 * (size_t)HID * OUTP);
     const size_t o_XT = take(2 * (size_t)IN * Bp);
-    size_t o_H[3], o_HT[3], o_Z[3], o_dZ[2], o_dZT[2], o_P[4];
+    size_t o_H[3], o_HT[3], o_Z[3], o_dZ[2], o_dZT[3], o_P[4];
     for (int l = 0; l < 3; ++l) {
         o_H[l] = take(2 * (size_t)Bp * HID);
         o_HT[l] = take(2 * (size_t)Bp * HID);
         o_Z[l] = take(4 * (size_t)Bp * HID);
     }
     const size_t o_dO = take(2 * (size_t)Bp * OUTP), o_dOT = take(2 * (size_t)Bp * OUTP);
-    for (int b = 0; b < 2; ++b) {
-        o_dZ[b] = take(2 * (size_t)Bp * HID);
-        o_dZT[b] = take(2 * (size_t)Bp * HID);
-    }
+    for (int b = 0; b < 2; ++b) o_dZ[b] = take(2 * (size_t)Bp * HID);
+    for (int l = 0; l < 3; ++l) o_dZT[l] = take(2 * (size_t)Bp * HID);
     o_P[0] = take(4 * (size_t)S * HID * IN);
     o_P[1] = take(4 * (size_t)S * HID * HID);
     o_P[2] = take(4 * (size_t)S * HID * HID);
@@ -1210,10 +1297,8 @@ int idm_mlp_create(idm_mlp_t **out, int32_t max_batch)
     }
     n->dO = (bf16 *)(a + o_dO);
     n->dOT = (bf16 *)(a + o_dOT);
-    for (int b = 0; b < 2; ++b) {
-        n->dZ[b] = (bf16 *)(a + o_dZ[b]);
-        n->dZT[b] = (bf16 *)(a + o_dZT[b]);
-    }
+    for (int b = 0; b < 2; ++b) n->dZ[b] = (bf16 *)(a + o_dZ[b]);
+    for (int l = 0; l < 3; ++l) n->dZT[l] = (bf16 *)(a + o_dZT[l]);
     n->db = (float *)(a + o_db);
     n->loss_part = (double *)(a + o_lp);
     n->loss_tmp = (double *)(a + o_lt);
@@ -1327,7 +1412,7 @@ int idm_mlp_features(const idm_scene_t *sc, const float *p_init, const float *v_
             f.hi[q] = box_hi[q];
         }
     }
-    idm::mlp::features_kernel<<<(n_rows + 127) / 128, 128, 0, (cudaStream_t)stream>>>(f);
+    idm::mlp::features_kernel<<<(n_rows + FEAT_THREADS - 1) / FEAT_THREADS, FEAT_THREADS, 0, (cudaStream_t)stream>>>(f);
     if (cudaGetLastError() != cudaSuccess) return IDM_ERR_CUDA;
     return IDM_OK;
 }
@@ -1352,7 +1437,7 @@ int idm_mlp_forward(idm_mlp_t *n, const void *X, int32_t B, float *out, void *st
     g.k_chunk = HID;
     g.bias = n->w + OFF_B4;
     g.out[0] = out;
-    MCK(gemm_batch<OUT_INFER>(g, n->n_sm, st));
+    MCK(gemm_batch<OUT_INFER>(g, n->n_sm, true, st));
     return IDM_OK;
 }
 
@@ -1390,7 +1475,7 @@ int idm_mlp_predict_params(idm_mlp_t *n, const void *X, int32_t B, idm_params_t 
             g.lo[q] = box_lo[q];
             g.hi[q] = box_hi[q];
         }
-        MCK(gemm_batch<OUT_INFER>(g, n->n_sm, st));
+        MCK(gemm_batch<OUT_INFER>(g, n->n_sm, true, st));
     }
     return IDM_OK;
 }
