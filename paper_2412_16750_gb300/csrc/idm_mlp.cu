@@ -721,6 +721,17 @@ __device__ __forceinline__ float obs_at(const FeatArgs &f, int i, int j)
     return j == 0 ? f.p_init[i] : f.targets[(size_t)(j - 1) * f.N + i];
 }
 
+// x / b for a constant b: the estimate by the rounded reciprocal corrected once
+// by its residual, which gives the correctly rounded quotient (P. Markstein,
+// "Computation of elementary functions on the IBM RISC System/6000 processor",
+// IBM J. Res. Dev. 34, 1990); an infinite or undefined estimate stands.
+__device__ __forceinline__ float div_const(float x, float b)
+{
+    const float rb = 1.0f / b, q = x * rb;  // rb: folded at compile time
+    const float c = fmaf(fmaf(-q, b, x), rb, q);
+    return isfinite(q) ? c : q;
+}
+
 // One thread per row; the block's rows are staged in shared memory (41 words a
 // row, so that the threads' words fall in different banks) and leave as one
 // contiguous run of words.  HBM-bound in principle (80 B in, 160 B out per
@@ -750,11 +761,11 @@ __global__ void __launch_bounds__(FEAT_THREADS) features_kernel(const FeatArgs f
         // words of the leader as well
         auto series = [&](int k, int w, bool virt) {
             float prev = obs_at(f, k, 0), cur = obs_at(f, k, 1);
-            float xa = (prev - y0) / 100.0f, va = f.v_init[k] / 30.0f;
+            float xa = div_const(prev - y0, 100.0f), va = div_const(f.v_init[k], 30.0f);
 #pragma unroll
             for (int j = 1; j < PREFIX; ++j) {
                 const float next = obs_at(f, k, j + 1);
-                const float x = (cur - y0) / 100.0f, v = (next - prev) * inv_2sdt / 30.0f;
+                const float x = div_const(cur - y0, 100.0f), v = div_const((next - prev) * inv_2sdt, 30.0f);
                 if (j & 1) {
                     const uint32_t vw = pack(va, v);
                     out[w + j / 2] = pack(xa, x);
