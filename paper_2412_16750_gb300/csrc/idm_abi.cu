@@ -235,10 +235,10 @@ static int prepare(idm_ctx *c, const idm_scene_t *sc, const idm_params_t *pr, co
     a.G = G;
     (void)need_loss;
 
-    CK(cudaMemsetAsync(c->ctl.p, 0, sizeof(int) * 3, st));
-    CK(idm::launch_prep_gap(sc->lane_off, L, p_init, sc->length, N, (float *)c->g0.p, a.status, st));
-    CK(idm::launch_build_segments(sc->lane_off, L, 32 * P->vpt * G, N, lanes_fit_one_wave(c, L, G),
-                                  (Seg *)c->seg.p, (int *)c->ctl.p + CTL_NSEG, a.status, st));
+    int *ctl = (int *)c->ctl.p;
+    CK(idm::launch_prep(sc->lane_off, L, p_init, sc->length, N, (float *)c->g0.p, 32 * P->vpt * G,
+                        lanes_fit_one_wave(c, L, G), (Seg *)c->seg.p, ctl + CTL_NSEG, ctl + CTL_WORK_F, ctl + CTL_WORK_B,
+                        a.status, st));
     P->loss_per_seg = G;
     P->k_max = sim->K;
     return forward_grid(c, P, L);
@@ -434,7 +434,7 @@ int run_fit_graph(idm_ctx *c, Prep &P, int n_iter, size_t N, const float *box_lo
             if (e == cudaSuccess && c->profiling) e = cudaEventRecordWithFlags(c->ev[4 * it + 3], cs, cudaEventRecordExternal);
             if (e == cudaSuccess) e = finalize(c, P, it, loss_hist, cs);  // loss of the parameters before update it
             if (e == cudaSuccess && eval)
-                e = idm::launch_loss_finalize((const double *)c->eval_part.p, a.n_seg, P.G_f, eval_hist + it, cs);
+                e = idm::launch_loss_finalize((const double *)c->eval_part.p, a.n_seg, P.G_f, 1024, eval_hist + it, cs);
         }
         cudaError_t e2 = cudaStreamEndCapture(cs, &g);
         if (e != cudaSuccess) { if (g) cudaGraphDestroy(g); return cuda_fail(c, e, "capturing the fit"); }
@@ -518,7 +518,7 @@ namespace {
 cudaError_t single_finalize(idm_ctx *c, const Prep &P, int it, double *hist, cudaStream_t st)
 {
     (void)c;
-    return idm::launch_loss_finalize(P.a.loss_part, P.a.n_seg, P.loss_per_seg, hist ? hist + it : nullptr, st);
+    return idm::launch_loss_finalize(P.a.loss_part, P.a.n_seg, P.loss_per_seg, 1024, hist ? hist + it : nullptr, st);
 }
 
 }  // namespace
@@ -758,7 +758,8 @@ int idm_loss_grad(idm_ctx_t *c, const idm_scene_t *scene, const idm_params_t *pa
     P.a.g_p_init = grad_p_init;
     P.a.g_v_init = grad_v_init;
     CK(idm::launch_backward(P.vpt, P.G, false, false, want_delta, P.a, P.grid_b, P.wpb_b, st));
-    CK(idm::launch_loss_finalize(P.a.loss_part, P.a.n_seg, P.G, loss_out ? loss_out : (double *)c->loss_tmp.p, st));
+    CK(idm::launch_loss_finalize(P.a.loss_part, P.a.n_seg, P.G, (long long)scene->n_lanes * P.G,
+                                 loss_out ? loss_out : (double *)c->loss_tmp.p, st));
     return IDM_OK;
 }
 

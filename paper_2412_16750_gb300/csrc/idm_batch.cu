@@ -219,7 +219,7 @@ cudaError_t batch_finalize(idm_ctx *c, const Prep &P, int it, double *hist, cuda
     if (g_bfin.scen_loss)
         scen_loss_kernel<<<(S + 255) / 256, 256, 0, st>>>(P.a.loss_part, P.loss_per_seg, (const int *)c->scen_seg_off.p,
                                                           (const int *)c->scen_seg_idx.p, S, g_bfin.scen_loss);
-    if (hist) return idm::launch_loss_finalize(P.a.loss_part, P.a.n_seg, P.loss_per_seg, hist + it, st);
+    if (hist) return idm::launch_loss_finalize(P.a.loss_part, P.a.n_seg, P.loss_per_seg, 1024, hist + it, st);
     return cudaGetLastError();
 }
 

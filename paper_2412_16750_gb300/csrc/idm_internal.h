@@ -113,7 +113,12 @@ size_t forward_smem_bytes(int vpt, int G, int wpb);
 int backward_max_warps(int vpt, int G);
 // Adjoint warps per SM the register budgets allow for a shape.
 int backward_resident_warps(int vpt, int G);
-cudaError_t launch_loss_finalize(const double *loss_part, const int *n_seg, int per_seg, double *out, cudaStream_t st);
+// max_part: at least the number of partials (n_seg * per_seg).
+cudaError_t launch_loss_finalize(const double *loss_part, const int *n_seg, int per_seg, long long max_part, double *out,
+                                 cudaStream_t st);
+// Initial gaps, work counters cleared and lanes packed into segments.
+cudaError_t launch_prep(const int *lane_off, int n_lanes, const float *p_init, const float *length, int N, float *g0, int cap,
+                        bool one_wave, Seg *seg, int *n_seg, int *work_f, int *work_b, unsigned *status, cudaStream_t st);
 // Single-launch fit (idm_fused.cuh): every Adam iteration of every segment
 // in one persistent launch of the adjoint's shape (vpt, G, wpb, tape depth
 // and prefetch of `a`); loss partial of iteration it at

@@ -198,12 +198,9 @@ extern "C" int idm_loss_grad_noalloc(const idm_scene_t *sc, const idm_params_t *
 
     // the array keeps the previous call's contents: clear counters and status
     if (cudaMemsetAsync(base, 0, o_seg, st) != cudaSuccess) return IDM_ERR_CUDA;
-    cudaError_t e = idm::launch_prep_gap(sc->lane_off, (int)L, p_init, sc->length, (int)N, (float *)(base + o_g0),
-                                         status, st);
-    if (e == cudaSuccess)
-        e = idm::launch_build_segments(sc->lane_off, (int)L, 32 * P.vpt * G, (int)N,
-                                       lanes_fit_one_wave(&c, (int)L, G), (Seg *)(base + o_seg),
-                                       ctl + CTL_NSEG, status, st);
+    cudaError_t e = idm::launch_prep(sc->lane_off, (int)L, p_init, sc->length, (int)N, (float *)(base + o_g0),
+                                     32 * P.vpt * G, lanes_fit_one_wave(&c, (int)L, G), (Seg *)(base + o_seg),
+                                     ctl + CTL_NSEG, ctl + CTL_WORK_F, ctl + CTL_WORK_B, status, st);
     if (e == cudaSuccess) {
         a.work = ctl + CTL_WORK_F;
         e = idm::launch_forward(P.vpt_f, P.G_f, false, false, true, a, P.grid_f, P.wpb_f, st);
@@ -219,7 +216,7 @@ extern "C" int idm_loss_grad_noalloc(const idm_scene_t *sc, const idm_params_t *
         e = idm::launch_backward(P.vpt, P.G, false, false, want_delta, a, P.grid_b, P.wpb_b, st);
     }
     if (e == cudaSuccess)
-        e = idm::launch_loss_finalize(a.loss_part, a.n_seg, G, loss_out ? loss_out : (double *)(base + o_loss), st);
+        e = idm::launch_loss_finalize(a.loss_part, a.n_seg, G, (long long)L * G, loss_out ? loss_out : (double *)(base + o_loss), st);
     if (e == cudaSuccess && status_out)
         e = cudaMemcpyAsync(status_out, status, sizeof(unsigned), cudaMemcpyDeviceToDevice, st);
     if (e != cudaSuccess) {

@@ -24,13 +24,21 @@ namespace idm {
 // Initial gaps g0[i] = p_init[i-1] - p_init[i] - length[i-1] (Sec. III-A),
 // +inf for lane heads.
 // ---------------------------------------------------------------------------
+__device__ __forceinline__ float initial_gap(const float *p_init, const float *length, int i)
+{
+    if (i == 0) return INFINITY;
+    return (float)((double)p_init[i - 1] - (double)p_init[i] - (double)length[i - 1]);
+}
+
+__device__ __forceinline__ bool bad_lane(int l, int a, int e, int n_lanes, int N)
+{
+    return e < a || a < 0 || e > N || (l == 0 && a != 0) || (l == n_lanes - 1 && e != N);
+}
+
 __global__ void gap_kernel(const float *p_init, const float *length, int N, float *g0)
 {
     int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= N) return;
-    if (i == 0) { g0[0] = INFINITY; return; }
-    double g = (double)p_init[i - 1] - (double)p_init[i] - (double)length[i - 1];
-    g0[i] = (float)g;
+    if (i < N) g0[i] = initial_gap(p_init, length, i);
 }
 
 __global__ void head_kernel(const int *lane_off, int n_lanes, int N, float *g0, unsigned *status)
@@ -38,8 +46,7 @@ __global__ void head_kernel(const int *lane_off, int n_lanes, int N, float *g0, 
     int l = blockIdx.x * blockDim.x + threadIdx.x;
     if (l >= n_lanes) return;
     int a = lane_off[l], e = lane_off[l + 1];
-    bool bad = e < a || a < 0 || e > N || (l == 0 && a != 0) || (l == n_lanes - 1 && e != N);
-    if (bad) { atomicOr(status, IDM_STATUS_BAD_LANE_OFF); return; }
+    if (bad_lane(l, a, e, n_lanes, N)) { atomicOr(status, IDM_STATUS_BAD_LANE_OFF); return; }
     if (a < e) g0[a] = INFINITY;
 }
 
@@ -100,13 +107,10 @@ __device__ int pack_lanes(const int *lane_off, int l0, int l1, int cap, int N, S
     return cnt;
 }
 
-__global__ void __launch_bounds__(BUILD_THREADS)
-build_segments_kernel(const int *lane_off, int n_lanes, int cap, int N, int per, bool staged, Seg *seg, int *n_seg,
-                      unsigned *status)
+__device__ __forceinline__ void build_segments(const int *lane_off, int n_lanes, int cap, int N, int per, bool staged,
+                                               Seg *seg, int *n_seg, unsigned *status, int *off, int *sc)
 {
-    extern __shared__ int off[];                                          // [n_lanes + 1] when staged
     unsigned short *jump = reinterpret_cast<unsigned short *>(off + n_lanes + 1);  // lanes of the segment from a lane
-    __shared__ int sc[BUILD_THREADS];
     const int t = threadIdx.x;
     const int l0 = (int)min((long long)n_lanes, (long long)t * per), l1 = min(n_lanes, l0 + per);
     if (staged) {
@@ -159,14 +163,78 @@ build_segments_kernel(const int *lane_off, int n_lanes, int cap, int N, int per,
     if (t == BUILD_THREADS - 1) *n_seg = sc[t];
 }
 
-cudaError_t launch_build_segments(const int *lane_off, int n_lanes, int cap, int N, bool one_wave, Seg *seg, int *n_seg,
-                                  unsigned *status, cudaStream_t st)
+__global__ void __launch_bounds__(BUILD_THREADS)
+build_segments_kernel(const int *lane_off, int n_lanes, int cap, int N, int per, bool staged, Seg *seg, int *n_seg,
+                      unsigned *status)
+{
+    extern __shared__ int off[];  // [n_lanes + 1] when staged, and the jumps
+    __shared__ int sc[BUILD_THREADS];
+    build_segments(lane_off, n_lanes, cap, N, per, staged, seg, n_seg, status, off, sc);
+}
+
+// The whole preparation in one launch, for scenes whose staged offsets leave
+// room for other blocks: block 0 clears the work counters, checks the lanes and
+// packs them; the others compute the initial gaps of 1,024 vehicles each, the
+// lane heads among them found in one pass over the offsets.  (A clear and three
+// kernels of 3-4 us each before a small scene's 75 us of simulation otherwise.)
+constexpr int FUSED_PREP_LANES = 4096;
+
+__global__ void __launch_bounds__(BUILD_THREADS)
+prep_kernel(const int *lane_off, int n_lanes, const float *p_init, const float *length, int N, float *g0, int cap, int per,
+            Seg *seg, int *ctl_nseg, int *work_f, int *work_b, unsigned *status)
+{
+    extern __shared__ int off[];
+    __shared__ int sc[BUILD_THREADS];
+    const int t = threadIdx.x;
+    if (blockIdx.x == 0) {
+        if (t == 0) *work_f = *work_b = 0;
+        for (int l = t; l < n_lanes; l += BUILD_THREADS)
+            if (bad_lane(l, lane_off[l], lane_off[l + 1], n_lanes, N)) atomicOr(status, IDM_STATUS_BAD_LANE_OFF);
+        build_segments(lane_off, n_lanes, cap, N, per, true, seg, ctl_nseg, status, off, sc);
+        return;
+    }
+    const int first = ((int)blockIdx.x - 1) * BUILD_THREADS, i = first + t;
+    sc[t] = 0;  // 1: a lane's head
+    __syncthreads();
+    for (int l = t; l < n_lanes; l += BUILD_THREADS) {
+        const int a = lane_off[l], e = lane_off[l + 1];
+        if (a < e && a >= first && a < first + BUILD_THREADS && !bad_lane(l, a, e, n_lanes, N)) sc[a - first] = 1;
+    }
+    __syncthreads();
+    if (i < N) g0[i] = sc[t] ? INFINITY : initial_gap(p_init, length, i);
+}
+
+// Lanes per chunk of the packing.
+static int lanes_per_chunk(int n_lanes, int cap, int N, bool one_wave)
 {
     // 32 segments of as many whole lanes of the mean length as fit
     const long long mean = N > 0 ? ((long long)N + n_lanes - 1) / n_lanes : 1;
     const long long full = 32 * (mean < cap ? cap / mean : 1), least = ((long long)n_lanes + BUILD_THREADS - 1) / BUILD_THREADS;
     const bool short_lanes = (long long)N < 16LL * n_lanes;
-    const int per = (int)(one_wave || short_lanes || full < least ? least : full);  // lanes per chunk
+    return (int)(one_wave || short_lanes || full < least ? least : full);
+}
+
+cudaError_t launch_prep(const int *lane_off, int n_lanes, const float *p_init, const float *length, int N, float *g0, int cap,
+                        bool one_wave, Seg *seg, int *n_seg, int *work_f, int *work_b, unsigned *status, cudaStream_t st)
+{
+    cudaError_t e;
+    if (n_lanes <= FUSED_PREP_LANES) {
+        const int blocks = 1 + (N + BUILD_THREADS - 1) / BUILD_THREADS;
+        prep_kernel<<<blocks, BUILD_THREADS, staged_bytes(n_lanes), st>>>(lane_off, n_lanes, p_init, length, N, g0, cap,
+                                                                          lanes_per_chunk(n_lanes, cap, N, one_wave), seg,
+                                                                          n_seg, work_f, work_b, status);
+        return cudaGetLastError();
+    }
+    if ((e = cudaMemsetAsync(work_f, 0, sizeof(int), st)) != cudaSuccess) return e;
+    if ((e = cudaMemsetAsync(work_b, 0, sizeof(int), st)) != cudaSuccess) return e;
+    if ((e = launch_prep_gap(lane_off, n_lanes, p_init, length, N, g0, status, st)) != cudaSuccess) return e;
+    return launch_build_segments(lane_off, n_lanes, cap, N, one_wave, seg, n_seg, status, st);
+}
+
+cudaError_t launch_build_segments(const int *lane_off, int n_lanes, int cap, int N, bool one_wave, Seg *seg, int *n_seg,
+                                  unsigned *status, cudaStream_t st)
+{
+    const int per = lanes_per_chunk(n_lanes, cap, N, one_wave);
     const bool staged = n_lanes <= STAGED_LANES;
     const size_t smem = staged ? staged_bytes(n_lanes) : 0;
     cudaError_t e = cudaFuncSetAttribute(build_segments_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -195,9 +263,14 @@ loss_finalize_kernel(const double *part, const int *n_seg, int per_seg, double *
     if (threadIdx.x == 0 && out) *out = sh[0];
 }
 
-cudaError_t launch_loss_finalize(const double *loss_part, const int *n_seg, int per_seg, double *out, cudaStream_t st)
+cudaError_t launch_loss_finalize(const double *loss_part, const int *n_seg, int per_seg, long long max_part, double *out,
+                                 cudaStream_t st)
 {
-    loss_finalize_kernel<<<1, 1024, 0, st>>>(loss_part, n_seg, per_seg, out);
+    // a power of two of threads that covers the partials gives the sum of 1,024
+    // (whose other terms are zeros) with fewer barriers
+    int threads = 32;
+    while (threads < 1024 && threads < max_part) threads <<= 1;
+    loss_finalize_kernel<<<1, threads, 0, st>>>(loss_part, n_seg, per_seg, out);
     return cudaGetLastError();
 }
 
