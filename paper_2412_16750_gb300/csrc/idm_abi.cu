@@ -282,7 +282,7 @@ int forward_grid(idm_ctx *c, Prep *P, int L)
     }
     const int warps_needed = L * G;  // segments <= lanes
     const int blocks_needed = (warps_needed + P->wpb_f - 1) / P->wpb_f;
-    int occ_f = idm::occupancy_blocks(P->vpt_f, G, false, false, false, false, P->wpb_f, 0);
+    const int occ_f = idm::forward_blocks_per_sm(P->vpt_f, G, P->wpb_f);
     P->grid_f = std::min(blocks_needed, c->n_sm * occ_f);
     P->grid_f = P->grid_f < 1 ? 1 : P->grid_f;
     return IDM_OK;
@@ -295,33 +295,41 @@ int backward_grid(idm_ctx *c, Prep *P, bool dense, bool adam, bool want_delta, i
     const int G = P->G;
     const size_t reg_cap = std::max(1, idm::backward_resident_warps(P->vpt, G) / G);  // groups per SM by registers
     auto groups_per_sm = [&](int T, bool pf) -> size_t {
-        const size_t b = idm::backward_smem_bytes(P->vpt, dense, T, G, G, pf);
+        const size_t b = idm::backward_smem_bytes(P->vpt, T, G, G, pf);
         return b > smem_max ? 0 : sm_smem / (b + 1024);
     };
     // tape depth: the checkpoint interval, or less when a deeper tape would
     // cost resident groups (blocks inside a checkpoint segment then restart
     // from sub-checkpoints written by an extra forward pass)
     const int C = P->a.C;  // the call's checkpoint interval (at most its longest horizon)
+    // ... and at most what the block's share of the tensor memory holds
+    const int full_warps = std::max(idm::backward_max_warps(P->vpt, G), G);
+    const int full_blocks = std::max(1, idm::backward_resident_warps(P->vpt, G) / full_warps);
     int T = C;
+    while (T > 1 && full_blocks * idm::tape_columns(P->vpt, T, full_warps) > idm::TMEM_COLS) --T;
     const size_t want = std::min(reg_cap, std::max<size_t>(groups_per_sm(1, false), 1));
     while (T > 1 && groups_per_sm(T, false) < want) --T;
     if (groups_per_sm(T, false) == 0)
         return fail(c, IDM_ERR_ARG, "adjoint tape does not fit shared memory for vpt %d x %d warps", P->vpt, G);
+    P->a.sub_ckpt = nullptr;
+    if (T < C) {
+        const size_t rows = (size_t)((C + T - 1) / T - 1);
+        const int rc = ensure(c, c->sub_ckpt, sizeof(float) * idm::STATE_ROWS * rows * (size_t)std::max(P->a.N_total, 1),
+                              "sub-checkpoints");
+        // no room for them: an interval that fits the chip as one tape runs so,
+        // with fewer groups per SM
+        if (rc == IDM_ERR_WORKSPACE && idm::tape_columns(P->vpt, C, G) <= idm::TMEM_COLS && groups_per_sm(C, false) > 0)
+            T = C;
+        else if (rc)
+            return rc;
+        else
+            P->a.sub_ckpt = (float *)c->sub_ckpt.p;
+    }
     // prefetching the next block doubles two stages; use it when it does not
     // cost a resident group per SM
     const bool pf = groups_per_sm(T, true) >= std::min(reg_cap, groups_per_sm(T, false));
     P->a.bwd_pf = pf ? 1 : 0;
     P->a.tape_T = T;
-    if (T < C) {
-        const size_t rows = (size_t)((C + T - 1) / T - 1);
-        int rc;
-        if ((rc = ensure(c, c->sub_ckpt, sizeof(float) * idm::STATE_ROWS * rows * (size_t)std::max(P->a.N_total, 1),
-                         "sub-checkpoints")))
-            return rc;
-        P->a.sub_ckpt = (float *)c->sub_ckpt.p;
-    } else {
-        P->a.sub_ckpt = nullptr;
-    }
     // compensated totals of the gradient sums (folded only past the window),
     // for the most segments the packing can produce (L: lanes of a single
     // scene, or the batch's segments)
@@ -335,16 +343,21 @@ int backward_grid(idm_ctx *c, Prep *P, bool dense, bool adam, bool want_delta, i
     } else {
         P->a.gsum = nullptr;
     }
-    const size_t per_group = idm::backward_smem_bytes(P->vpt, dense, T, G, G, pf);
-    int groups = std::max(1, std::min(c->wpb / G, (int)(smem_max / per_group)));
+    const size_t per_group = idm::backward_smem_bytes(P->vpt, T, G, G, pf);
+    // at least four warps: a block of fewer leaves lane quarters of its tensor
+    // memory unused, and fewer blocks would fit an SM
+    int groups = std::max(1, std::min(std::max(c->wpb, 4) / G, (int)(smem_max / per_group)));
     groups = std::max(1, std::min(groups, idm::backward_max_warps(P->vpt, G) / G));
     // few segments: spread over the SMs (in blocks of whole quarters of warps)
     int spread = (int)((expected_segments(P->a.N_total, L, 32 * P->vpt * G) + c->n_sm - 1) / c->n_sm);
     if (spread * G > 4) spread = ((spread * G + 3) / 4 * 4 + G - 1) / G;
     groups = std::min(groups, spread);
+    while (groups > 1 && idm::tape_columns(P->vpt, T, groups * G) > idm::TMEM_COLS) --groups;
     P->wpb_b = groups * G;
     size_t smem = per_group * groups;
-    int occ_b = idm::occupancy_blocks(P->vpt, G, true, dense, adam, want_delta, P->wpb_b, smem, T < C);
+    P->a.tape_cols = idm::tape_columns(P->vpt, T, P->wpb_b);
+    const int occ_b =
+        idm::backward_blocks_per_sm(P->vpt, G, dense, adam, want_delta, P->wpb_b, smem, T < C, P->a.tape_cols);
     int blocks_needed = (L * G + P->wpb_b - 1) / P->wpb_b;
     P->grid_b = std::min(blocks_needed, c->n_sm * occ_b);
     P->grid_b = P->grid_b < 1 ? 1 : P->grid_b;

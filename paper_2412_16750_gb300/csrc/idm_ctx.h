@@ -28,7 +28,7 @@ struct Prep {
     int G_f = 1;
     int wpb_f = 1;  // warps per block of the forward (a multiple of G_f)
     int grid_f = 1, grid_b = 1;
-    int wpb_b = 1;  // warps per block of the adjoint (bounded by its shared-memory tape)
+    int wpb_b = 1;  // warps per block of the adjoint (bounded by its tape)
     int loss_per_seg = 1;
     int k_max = 0;  // longest horizon of the call (steps)
     SimArgs a;

@@ -66,6 +66,8 @@ __device__ __forceinline__ f2 rcp2(f2 x) { return make_float2(rcp_approx(x.x), r
 __device__ __forceinline__ f2 vmax(f2 a, f2 b) { return make_float2(fmaxf(a.x, b.x), fmaxf(a.y, b.y)); }
 __device__ __forceinline__ f2 vabs(f2 a) { return make_float2(fabsf(a.x), fabsf(a.y)); }
 
+__device__ __forceinline__ f2 neg2(f2 a) { return make_float2(-a.x, -a.y); }
+
 // Softplus pieces: e = exp(-|x|) = 2^(-|x| log2 e) and
 // sp(x) = max(x, 0) + ln(1 + e) = log2(1 + e) * ln 2 + max(x, 0).
 struct Soft2 {
@@ -128,19 +130,32 @@ __device__ __forceinline__ f2 lower_bound(f2 lbv, float a_min, bool &bx, bool &b
     return vmax(lbv, F2(a_min));  // equal values give a_min either way
 }
 
-// Bounded acceleration a* of two vehicles from their speeds v, raw gaps
-// (p_h - p - length_h; +inf for a lane head) and leaders' speeds vh.
+// 1 - r^delta - z^2 of Eq. 2.  The products are fused explicitly, so that the
+// forward and the adjoint's recompute round alike whatever else uses them.
 template <bool D4>
-__device__ __forceinline__ f2 accel_star2(f2 v, f2 gap_raw, f2 vh, const VehConst2 &k, float inv_dt, float a_min)
+__device__ __forceinline__ f2 free_minus_z2(f2 r, f2 z, f2 delta)
+{
+    f2 t;
+    if (D4) {
+        const f2 r2 = mul2(r, r);
+        t = fma2(neg2(r2), r2, F2(1.0f));
+    } else {
+        t = sub2(F2(1.0f), pow_delta2<false>(r, delta));
+    }
+    return fma2(neg2(z), z, t);
+}
+
+// Bounded acceleration a* of two vehicles from their speeds v, raw gaps
+// (p_h - p - length_h; +inf for a lane head) and speed differences dv to
+// their leaders (Sec. III-A).
+template <bool D4>
+__device__ __forceinline__ f2 accel_star2(f2 v, f2 gap_raw, f2 dv, const VehConst2 &k, float inv_dt, float a_min)
 {
     const f2 gap = floor_gap(gap_raw);
-    const f2 dv = sub2(v, vh);                                  // Sec. III-A
     const f2 s_opt = fma2(v, fma2(dv, k.c, k.T), k.s0);         // Eq. 1
     const Soft2 s1 = softplus2(s_opt);                          // Sec. III-C
     const f2 z = mul2(s1.sp, rcp2(gap));                        // 0 for a head
-    const f2 r = mul2(v, k.inv_v0);
-    const f2 rd = pow_delta2<D4>(r, k.delta);
-    const f2 a = mul2(k.am, sub2(sub2(F2(1.0f), rd), mul2(z, z)));  // Eq. 2
+    const f2 a = mul2(k.am, free_minus_z2<D4>(mul2(v, k.inv_v0), z, k.delta));  // Eq. 2
     bool bx, by;
     const f2 a_lb = lower_bound(mul2(v, F2(-inv_dt)), a_min, bx, by);  // Sec. III-C
     const Soft2 s2 = softplus2(sub2(a, a_lb));
@@ -169,8 +184,9 @@ struct State2 {
 // |ph| >= |d| (a step is at most a few metres); in the one or two steps in
 // which a vehicle passes within |d| of position 0 it is off by at most half
 // an ulp of the sum (~5e-7 m), three operations fewer per step than TwoSum.
-// The speed takes dt a* by Kahan's compensated summation.
-__device__ __forceinline__ void euler2(State2 &s, f2 a_star, f2 vh, f2 vch, float dt)
+// The speed takes dt a* by Kahan's compensated summation.  dv and dvc: own
+// minus leader's running sum and compensation.
+__device__ __forceinline__ void euler2(State2 &s, f2 a_star, f2 dv, f2 dvc, float dt)
 {
     const f2 d = mul2(F2(dt), s.v);
     const f2 en = fma2(F2(-dt), s.v, d);
@@ -178,7 +194,7 @@ __device__ __forceinline__ void euler2(State2 &s, f2 a_star, f2 vh, f2 vch, floa
     const f2 err = sub2(d, sub2(t, s.ph));
     s.ph = t;
     s.pl = fma2(F2(-dt), s.vc, add2(s.pl, sub2(err, en)));
-    s.gap = fma2(F2(dt), add2(sub2(vh, s.v), sub2(s.vc, vch)), s.gap);
+    s.gap = fma2(F2(dt), sub2(dvc, dv), s.gap);
     const f2 y = sub2(mul2(F2(dt), a_star), s.vc);
     const f2 tv = add2(s.v, y);
     s.vc = sub2(sub2(tv, s.v), y);
@@ -195,69 +211,99 @@ __device__ __forceinline__ f2 residual2(const State2 &s, f2 y) { return add2(sub
 __device__ __forceinline__ f2 position2(const State2 &s) { return add2(s.ph, s.pl); }
 
 // ---- neighbours in the warp's slot mapping -----------------------------------
-// Pair p of lane l holds the consecutive slots 64p + 2l (.x) and 64p + 2l + 1
-// (.y).  The leader of .y is the same thread's .x; the leader of .x is lane
-// l-1's .y (for lane 0: lane 31's .y of pair p-1, or lead_in for p = 0, the
-// previous warp's last slot or 0 at a segment start).
-template <int NP>
-__device__ __forceinline__ void leader_vals2(const f2 (&x)[NP], f2 (&out)[NP], int lane, float lead_in)
+// Two mappings of a warp's 64 NP slots to the pairs of its lanes, both with the
+// two slots of a pair adjacent, so that the leader of .y is the same pair's .x:
+//   interleaved (the forward's, whose trajectory rows then leave in runs of 64):
+//     pair p of lane l holds slots 64p + 2l and 64p + 2l + 1, and the leader of
+//     .x is lane l-1's .y (for lane 0: lane 31's .y of pair p-1);
+//   consecutive (CONSEC, the adjoint of dense seeds and a scene's fit): lane l
+//     holds slots 2 NP l ... 2 NP l + 2 NP - 1, so one shuffle serves all pairs
+//     of a lane and its shared tape rows are one 16-byte access.
+// For the warp's first slot the leader value is lead_in (the previous warp's
+// last slot, or 0 at a segment start).
+template <int NP, bool CONSEC>
+__device__ __forceinline__ int pair_slot(int p, int lane)
 {
-    float ry[NP];
+    return CONSEC ? 2 * NP * lane + 2 * p : 64 * p + 2 * lane;
+}
+
+// x minus the leader's x, per slot.
+template <int NP, bool CONSEC>
+__device__ __forceinline__ void minus_leader2(const f2 (&x)[NP], f2 (&out)[NP], int lane, float lead_in)
+{
+    float hx[NP];  // leader of each .x
+    if (CONSEC) {
+        const float up = __shfl_sync(FULL, x[NP - 1].y, (lane + 31) & 31);
+        hx[0] = lane == 0 ? lead_in : up;
 #pragma unroll
-    for (int p = 0; p < NP; ++p) ry[p] = __shfl_sync(FULL, x[p].y, (lane + 31) & 31);
+        for (int p = 1; p < NP; ++p) hx[p] = x[p - 1].y;
+    } else {
+        float ry[NP];
+#pragma unroll
+        for (int p = 0; p < NP; ++p) ry[p] = __shfl_sync(FULL, x[p].y, (lane + 31) & 31);
+#pragma unroll
+        for (int p = 0; p < NP; ++p) hx[p] = lane == 0 ? (p > 0 ? ry[p - 1] : lead_in) : ry[p];
+    }
 #pragma unroll
     for (int p = 0; p < NP; ++p) {
-        const float prev = p > 0 ? ry[p - 1] : lead_in;
-        out[p].x = lane == 0 ? prev : ry[p];
-        out[p].y = x[p].x;
+        // with every pair's .x leader a shuffled value the packed form is
+        // cheaper; else its operand pair would have to be built by moves
+        if (CONSEC)
+            out[p] = make_float2(__fsub_rn(x[p].x, hx[p]), __fsub_rn(x[p].y, x[p].x));
+        else
+            out[p] = sub2(x[p], make_float2(hx[p], x[p].x));
     }
 }
 
-// Follower values: the follower of .x is the same thread's .y; the follower
-// of .y is lane l+1's .x (for lane 31: lane 0's .x of pair p+1, or fin for the
-// warp's last slot).
-template <int NP>
-__device__ __forceinline__ void follower_vals2(const f2 (&x)[NP], f2 (&out)[NP], int lane, float fin)
+// x plus y's value of the follower, per slot: the follower of .x is the same
+// pair's .y, of .y the next slot's .x (fin for the warp's last slot).
+template <int NP, bool CONSEC>
+__device__ __forceinline__ void add_follower2(f2 (&x)[NP], const f2 (&y)[NP], int lane, float fin)
 {
-    float rx[NP];
+    float nx[NP];  // follower of each .y
+    if (CONSEC) {
+        const float dn = __shfl_sync(FULL, y[0].x, (lane + 1) & 31);
 #pragma unroll
-    for (int p = 0; p < NP; ++p) rx[p] = __shfl_sync(FULL, x[p].x, (lane + 1) & 31);
+        for (int p = 0; p + 1 < NP; ++p) nx[p] = y[p + 1].x;
+        nx[NP - 1] = lane == 31 ? fin : dn;
+    } else {
+        float rx[NP];
 #pragma unroll
-    for (int p = 0; p < NP; ++p) {
-        const float nxt = p + 1 < NP ? rx[p + 1] : fin;
-        out[p].x = x[p].y;
-        out[p].y = lane == 31 ? nxt : rx[p];
+        for (int p = 0; p < NP; ++p) rx[p] = __shfl_sync(FULL, y[p].x, (lane + 1) & 31);
+#pragma unroll
+        for (int p = 0; p < NP; ++p) nx[p] = lane == 31 ? (p + 1 < NP ? rx[p + 1] : fin) : rx[p];
     }
+#pragma unroll
+    for (int p = 0; p < NP; ++p) x[p] = make_float2(__fadd_rn(x[p].x, y[p].y), __fadd_rn(x[p].y, nx[p]));
 }
 
 // ---- adjoint coefficients ------------------------------------------------------
-// Coefficients of one reverse step for a vehicle pair (the adjoint of
-// accel_star2 and euler2), independent of the incoming adjoint.  With
-// sigma2 = d a*/d a, sigma1 = d s*/d s_opt, Sn = -d a/d s* = 2 a_max z / gap
-// and G = d a/d gap = Sn z (0 below the gap floor):
+// One step's bounded acceleration and the coefficients of its reverse step,
+// for a vehicle pair (the adjoint of accel_star2 and euler2).  With sigma2 =
+// d a*/d a, sigma1 = d s*/d s_opt, Sn = -d a/d s* = 2 a_max z / gap and G =
+// d a/d gap = Sn z (0 below the gap floor):
 //   Aph = d a*/d p_leader  =  sigma2 G  (own d a*/d p is -Aph)
-//   Av  = d a*/d v         (own speed, incl. the a_lb branch)
-//   Avh = d a*/d v_leader  =  w0n c v,  w0n = sigma2 Sn sigma1
+//   Avn = -d a*/d v        (own speed, incl. the a_lb branch)
+//   w0n = sigma2 Sn sigma1 (d a*/d v_leader = w0n c v)
 // and the parameter-gradient factors, all sign-positive forms (per-vehicle
-// constants and signs are applied once at the end): w0n, w0n v, w0n v dv,
-// sigma2 (1 - r^delta - z^2), sigma2 r^delta, sigma2 r^delta ln r.  The
-// reverse step multiplies all of them by mu = dt * (adjoint of the
-// step-(k+1) speed).
-struct AdjJac2 {
-    f2 Aph, Av, Avh;
-    f2 w0n, w0nv, w0nvdv, fa, frd, frdl;
+// constants and signs are applied once at the end): w0n, w0n v, w0n v dv
+// (from w0n and the speeds), fa = sigma2 (1 - r^delta - z^2), frd = sigma2
+// r^delta, sigma2 r^delta ln r (from frd and v).  The reverse step multiplies
+// all of them by mu = dt * (adjoint of the step-(k+1) speed).
+struct StepJac2 {
+    f2 Aph, Avn, w0n, fa, frd;
 };
 
-// qc: with D4, the per-vehicle constant 4 a_max / v0 of the free-road term's
-// speed derivative (ignored otherwise).
-template <bool WANT_DELTA, bool D4>
-__device__ __forceinline__ AdjJac2 adjoint_jac2(f2 v, f2 gap_raw, f2 vh, const VehConst2 &k, float inv_dt,
-                                                float a_min, f2 qc = F2(0.0f))
+// The acceleration is accel_star2's, operation for operation, so the adjoint's
+// recompute follows the forward bit for bit; the coefficients share its
+// softplus, reciprocal and power terms.  qc: with D4, the per-vehicle constant
+// 4 a_max / v0 of the free-road term's speed derivative (ignored otherwise).
+template <bool D4>
+__device__ __forceinline__ f2 accel_jac2(f2 v, f2 gap_raw, f2 dv, const VehConst2 &k, float inv_dt, float a_min,
+                                         f2 qc, StepJac2 &J)
 {
-    AdjJac2 J;
     const bool fx = gap_raw.x < IDM_GAP_FLOOR, fy = gap_raw.y < IDM_GAP_FLOOR;
     const f2 gap = floor_gap(gap_raw);
-    const f2 dv = sub2(v, vh);
     const f2 s_opt = fma2(v, fma2(dv, k.c, k.T), k.s0);
     const Soft2 s1 = softplus2(s_opt);
     // sigma(s_opt) = exp(s_opt - sp(s_opt)): the exponent is <= 0 and carries
@@ -277,11 +323,12 @@ __device__ __forceinline__ AdjJac2 adjoint_jac2(f2 v, f2 gap_raw, f2 vh, const V
             r.x > 0.0f ? __powf(r.x, k.delta.x - 1.0f) : (k.delta.x > 1.0f ? 0.0f : (k.delta.x == 1.0f ? 1.0f : INFINITY)),
             r.y > 0.0f ? __powf(r.y, k.delta.y - 1.0f) : (k.delta.y > 1.0f ? 0.0f : (k.delta.y == 1.0f ? 1.0f : INFINITY)));
     }
-    const f2 free_and_int = sub2(sub2(F2(1.0f), rd), mul2(z, z));
-    const f2 a = mul2(k.am, free_and_int);
     bool bx, by;
     const f2 a_lb = lower_bound(mul2(v, F2(-inv_dt)), a_min, bx, by);
-    const f2 x2 = sub2(a, a_lb);
+    const Soft2 s2 = softplus2(sub2(mul2(k.am, free_minus_z2<D4>(r, z, k.delta)), a_lb));
+    // the coefficients take 1 - r^delta from the rounded r^delta that frd needs
+    const f2 free_and_int = fma2(neg2(z), z, sub2(F2(1.0f), rd));
+    const f2 x2 = sub2(mul2(k.am, free_and_int), a_lb);
     const f2 e2 = make_float2(ex2_approx(fabsf(x2.x) * -LOG2E), ex2_approx(fabsf(x2.y) * -LOG2E));
     f2 sig2, one_m_sig2;
     sigmoid2(x2, e2, sig2, one_m_sig2);
@@ -290,32 +337,33 @@ __device__ __forceinline__ AdjJac2 adjoint_jac2(f2 v, f2 gap_raw, f2 vh, const V
     f2 G = mul2(Sn, z);                                          // d a / d gap = 2 a_max z^2 / gap
     G.x = fx ? 0.0f : G.x;
     G.y = fy ? 0.0f : G.y;
-    const f2 w0n = mul2(mul2(sig2, Sn), sig1);
+    J.w0n = mul2(mul2(sig2, Sn), sig1);
     const f2 q = D4 ? mul2(qc, rdm1) : mul2(mul2(k.am, k.delta), mul2(rdm1, k.inv_v0));  // -d(free term)/dv
     f2 beta_term = mul2(one_m_sig2, F2(inv_dt));
     beta_term.x = bx ? beta_term.x : 0.0f;
     beta_term.y = by ? beta_term.y : 0.0f;
     J.Aph = mul2(sig2, G);
     const f2 u = fma2(k.c, add2(v, dv), k.T);                    // d s_opt / d v
-    J.Av = mul2(fma2(sig2, q, fma2(w0n, u, beta_term)), F2(-1.0f));
-    J.Avh = mul2(mul2(w0n, k.c), v);
-    J.w0n = w0n;
-    J.w0nv = mul2(w0n, v);
-    J.w0nvdv = mul2(J.w0nv, dv);
+    J.Avn = fma2(sig2, q, fma2(J.w0n, u, beta_term));
     J.fa = mul2(sig2, free_and_int);
     J.frd = mul2(sig2, rd);
-    if (WANT_DELTA) {
-        const f2 lnr = mul2(lg2(r), F2(LN2));
-        const f2 t = mul2(J.frd, lnr);
-        // r^delta ln r -> 0 as r -> 0+.  Near rest the a_lb = -v/dt branch
-        // leaves v + dt a* within rounding of 0: a speed a few ulps below 0,
-        // or a denormal that the flush-to-zero logarithm reads as 0, also
-        // take the limit (r^delta has underflowed to 0 there)
-        J.frdl = make_float2(r.x > 0.0f && rd.x > 0.0f ? t.x : 0.0f, r.y > 0.0f && rd.y > 0.0f ? t.y : 0.0f);
-    } else {
-        J.frdl = F2(0.0f);
-    }
-    return J;
+    return add2(a_lb, s2.sp);
+}
+
+// sigma2 r^delta ln r of a step from its speed and frd = sigma2 r^delta.
+// r^delta ln r -> 0 as r -> 0+.  Near rest the a_lb = -v/dt branch leaves v +
+// dt a* within rounding of 0: a speed a few ulps below 0, or a denormal that
+// the flush-to-zero logarithm reads as 0, take the limit too: r^delta has
+// (all but) underflowed there, and with D4 the logarithm's argument is held
+// above 1e-37, so that the product is 0 to 1e-20.
+template <bool D4>
+__device__ __forceinline__ f2 delta_factor2(f2 v, f2 frd, const VehConst2 &k)
+{
+    const f2 r = mul2(v, k.inv_v0);
+    if (D4) return mul2(frd, mul2(lg2(vmax(r, F2(1e-37f))), F2(LN2)));
+    const f2 rd = pow_delta2<D4>(r, k.delta);
+    const f2 t = mul2(frd, mul2(lg2(r), F2(LN2)));
+    return make_float2(r.x > 0.0f && rd.x > 0.0f ? t.x : 0.0f, r.y > 0.0f && rd.y > 0.0f ? t.y : 0.0f);
 }
 
 }  // namespace idm

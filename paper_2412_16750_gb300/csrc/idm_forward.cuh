@@ -20,7 +20,7 @@ struct FwdFlags {
 // COUNT: also count the vehicle-steps with the raw gap below the floor and
 // those within IDM_KINK_BAND of the kink of the lower bound into a.events
 // (a separate instantiation, so the plain forward carries no cost of it).
-template <int NP, bool D4, bool COUNT = false>
+template <int NP, bool D4, bool CONSEC, bool COUNT = false>
 __device__ __forceinline__ void forward_segment(const SimArgs &a, const ScenDesc &sc, int s_idx, int lb, Grp &g,
                                                 const VehConst2 (&kc)[NP], State2 (&st)[NP], const bool (&vx)[NP],
                                                 const bool (&vy)[NP], FwdFlags f)
@@ -38,7 +38,7 @@ __device__ __forceinline__ void forward_segment(const SimArgs &a, const ScenDesc
             float *base = a.ckpt + sc.ckpt_off + (size_t)ck_idx * STATE_ROWS * Ns + wl;
 #pragma unroll
             for (int p = 0; p < NP; ++p) {
-                const int q = 64 * p + 2 * lane;
+                const int q = pair_slot<NP, CONSEC>(p, lane);
                 store_pair(base, q, st[p].ph, vx[p], vy[p]);
                 store_pair(base + (size_t)Ns, q, st[p].pl, vx[p], vy[p]);
                 store_pair(base + 2 * (size_t)Ns, q, st[p].v, vx[p], vy[p]);
@@ -52,7 +52,7 @@ __device__ __forceinline__ void forward_segment(const SimArgs &a, const ScenDesc
             const size_t row = sc.traj_off + (size_t)k * Ns + wl;
 #pragma unroll
             for (int p = 0; p < NP; ++p) {
-                const int q = 64 * p + 2 * lane;
+                const int q = pair_slot<NP, CONSEC>(p, lane);
                 if (f.traj) store_pair(a.traj + row, q, position2(st[p]), vx[p], vy[p]);
                 if (f.vtraj) store_pair(a.vtraj + row, q, speed2(st[p]), vx[p], vy[p]);
             }
@@ -63,7 +63,7 @@ __device__ __forceinline__ void forward_segment(const SimArgs &a, const ScenDesc
                 f2 e = F2(0.0f);
 #pragma unroll
                 for (int p = 0; p < NP; ++p) {
-                    f2 r = residual2(st[p], load_pair(y, 64 * p + 2 * lane, vx[p], vy[p]));
+                    f2 r = residual2(st[p], load_pair(y, pair_slot<NP, CONSEC>(p, lane), vx[p], vy[p]));
                     r.x = vx[p] ? r.x : 0.0f;
                     r.y = vy[p] ? r.y : 0.0f;
                     e = fma2(r, r, e);
@@ -86,7 +86,7 @@ __device__ __forceinline__ void forward_segment(const SimArgs &a, const ScenDesc
             }
         }
 
-        step_pairs<NP, D4>(g, st, kc, sc, xp);
+        step_pairs<NP, D4, CONSEC>(g, st, kc, sc, xp);
     }
     bool bad = false;
 #pragma unroll
@@ -134,11 +134,11 @@ forward_kernel(SimArgs a, FwdFlags f)
         VehConst2 kc[NP];
         State2 st[NP];
         bool vx[NP], vy[NP];
-        load_vehicles<NP>(a, sg, g.lane, g.w * 64 * NP, kc, st, vx, vy);
+        load_vehicles<NP, false>(a, sg, g.lane, g.w * 64 * NP, kc, st, vx, vy);
         if (segment_is_d4<NP>(kc, vx, vy))
-            forward_segment<NP, true, COUNT>(a, sc, s_idx, lb, g, kc, st, vx, vy, f);
+            forward_segment<NP, true, false, COUNT>(a, sc, s_idx, lb, g, kc, st, vx, vy, f);
         else
-            forward_segment<NP, false, COUNT>(a, sc, s_idx, lb, g, kc, st, vx, vy, f);
+            forward_segment<NP, false, false, COUNT>(a, sc, s_idx, lb, g, kc, st, vx, vy, f);
     }
 }
 

@@ -24,15 +24,15 @@
 
 namespace idm {
 
-template <int VPT, int GW, bool SUB>
+template <int VPT, int GW, bool SUB, bool CONSEC>
 __global__ void __launch_bounds__(BwdBounds<VPT, GW>::threads, BwdBounds<VPT, GW>::blocks)
 fit_fused_kernel(SimArgs a, long long part_stride)
 {
     constexpr int NP = VPT / 2;
     constexpr int G = GW;
-    extern __shared__ float smem[];
+    extern __shared__ __align__(16) float smem[];
     const int warp = threadIdx.x >> 5;
-    const int gf = bwd_group_floats(VPT, false, a.tape_T, G, a.bwd_pf != 0);
+    const int gf = bwd_group_floats(VPT, a.tape_T, G, a.bwd_pf != 0);
     float *gbase = smem + (warp / G) * gf;
     float *ctrl = gbase + gf - grp_ctrl_floats(G);
     Grp g = make_grp(G, ctrl);
@@ -44,6 +44,8 @@ fit_fused_kernel(SimArgs a, long long part_stride)
         if (threadIdx.x == 0) atomicOr(a.status, IDM_STATUS_LANE_TOO_LONG);
         return;
     }
+    const uint32_t tmem = tape_alloc(a.tape_cols);
+    const uint32_t tape = tape_base(tmem, warp, TAPE_WORDS * VPT * a.tape_T);
     double *const part0 = a.loss_part;
     const FwdFlags ff{false, false, true, false};
     int par = 0;
@@ -59,7 +61,7 @@ fit_fused_kernel(SimArgs a, long long part_stride)
             VehConst2 kc[NP];
             State2 st[NP], sf[NP];
             bool vx[NP], vy[NP];
-            load_vehicles<NP>(a, sg, g.lane, g.w * 64 * NP, kc, st, vx, vy);
+            load_vehicles<NP, CONSEC>(a, sg, g.lane, g.w * 64 * NP, kc, st, vx, vy);
             const bool d4 = segment_is_d4<NP>(kc, vx, vy);
 #pragma unroll
             for (int p = 0; p < NP; ++p) sf[p] = st[p];
@@ -67,33 +69,35 @@ fit_fused_kernel(SimArgs a, long long part_stride)
             // initial state: written in the first iteration, unchanged after
             if (it == 0 || sc.K > a.C) {
                 if (d4)
-                    forward_segment<NP, true>(a, sc, s_idx, lb, g, kc, sf, vx, vy, ff);
+                    forward_segment<NP, true, CONSEC>(a, sc, s_idx, lb, g, kc, sf, vx, vy, ff);
                 else
-                    forward_segment<NP, false>(a, sc, s_idx, lb, g, kc, sf, vx, vy, ff);
+                    forward_segment<NP, false, CONSEC>(a, sc, s_idx, lb, g, kc, sf, vx, vy, ff);
                 __threadfence_block();
                 grp_sync(g);  // the group's exchange cells: the forward's last reads before the adjoint's first writes
             }
             if constexpr (SUB) {
                 if (d4)
-                    backward_segment_blocks<NP, false, true, false, true>(a, sc, sg, s_idx, lb, g, gbase, kc, st, vx, vy);
+                    backward_segment_blocks<NP, false, true, false, true, CONSEC>(a, sc, sg, s_idx, lb, g, gbase, tape, kc, st);
                 else
-                    backward_segment_blocks<NP, false, true, false, false>(a, sc, sg, s_idx, lb, g, gbase, kc, st, vx,
-                                                                           vy);
+                    backward_segment_blocks<NP, false, true, false, false, CONSEC>(a, sc, sg, s_idx, lb, g, gbase, tape, kc, st);
             } else {
                 if (d4)
-                    backward_segment<NP, false, true, false, true>(a, sc, sg, s_idx, lb, g, gbase, kc, st, vx, vy);
+                    backward_segment<NP, false, true, false, true, CONSEC>(a, sc, sg, s_idx, lb, g, gbase, tape, kc, st);
                 else
-                    backward_segment<NP, false, true, false, false>(a, sc, sg, s_idx, lb, g, gbase, kc, st, vx, vy);
+                    backward_segment<NP, false, true, false, false, CONSEC>(a, sc, sg, s_idx, lb, g, gbase, tape, kc, st);
             }
             grp_sync(g);  // and the adjoint's last reads before the next forward's first writes
         }
     }
+    tape_free(tmem, a.tape_cols);
 }
 
 template <int VPT, int GW>
-inline void *fused_fn_t(bool sub)
+inline void *fused_fn_t(bool sub, bool consec)
 {
-    return sub ? (void *)fit_fused_kernel<VPT, GW, true> : (void *)fit_fused_kernel<VPT, GW, false>;
+    if (consec || VPT == 2)
+        return sub ? (void *)fit_fused_kernel<VPT, GW, true, true> : (void *)fit_fused_kernel<VPT, GW, false, true>;
+    return sub ? (void *)fit_fused_kernel<VPT, GW, true, VPT == 2> : (void *)fit_fused_kernel<VPT, GW, false, VPT == 2>;
 }
 
 // The forward, adjoint and single-launch fit kernels of one shape, as the
@@ -101,10 +105,11 @@ inline void *fused_fn_t(bool sub)
 // the shapes compile in parallel).
 #define IDM_DEFINE_SHAPE_KERNELS(V, GW)                                                  \
     void *forward_fn_v##V##_g##GW(bool count) { return forward_fn_t<V, GW>(count); }     \
-    void *backward_fn_v##V##_g##GW(bool dense, bool adam, bool wd, bool sub)              \
+    void *backward_fn_v##V##_g##GW(bool dense, bool adam, bool wd, bool sub, bool consec) \
     {                                                                                    \
-        return sub ? backward_fn_t<V, GW, true>(dense, adam, wd) : backward_fn_t<V, GW, false>(dense, adam, wd); \
+        return sub ? backward_fn_t<V, GW, true>(dense, adam, wd, consec)                  \
+                   : backward_fn_t<V, GW, false>(dense, adam, wd, consec);                \
     }                                                                                    \
-    void *fused_fn_v##V##_g##GW(bool sub) { return fused_fn_t<V, GW>(sub); }
+    void *fused_fn_v##V##_g##GW(bool sub, bool consec) { return fused_fn_t<V, GW>(sub, consec); }
 
 }  // namespace idm

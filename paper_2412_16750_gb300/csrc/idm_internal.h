@@ -52,8 +52,10 @@ struct SimArgs {
     double *loss_part;          // [n_seg * G] per-warp loss
     float *ckpt;
     int C;                      // checkpoint interval (steps)
+    int loss_split;             // > 0: the horizon's one run sums the loss of the steps before it apart
     int tape_T;                 // adjoint tape depth (steps, <= C); tape_T < C uses sub_ckpt
-    float *sub_ckpt;            // [ceil(C/tape_T)-1][4][N_total] states inside a checkpoint segment
+    int tape_cols;              // tensor-memory columns of an adjoint block's tapes
+    float *sub_ckpt;            // [ceil(C/tape_T)-1][STATE_ROWS][N_total] states inside a checkpoint segment
     unsigned *status;
     // adjoint
     const float *gP, *gV;       // dense trajectory gradients (scenario-local time-major)
@@ -89,6 +91,19 @@ struct SimArgs {
 inline size_t gsum_bytes(size_t n_seg, int capacity) { return n_seg * (size_t)capacity * 12 * sizeof(float); }
 constexpr int GSUM_FOLD_STEPS = 256;
 
+// Tensor-memory words per vehicle and step of the adjoint's tape, and the
+// columns that a block of `warps` warps allocates for a tape of T steps (a
+// power of two; the warps of a lane quarter, every fourth, sit side by side).
+constexpr int TAPE_WORDS = 4;
+constexpr int TMEM_COLS = 512;  // per SM
+inline int tape_columns(int vpt, int T, int warps)
+{
+    const int need = (warps + 3) / 4 * TAPE_WORDS * vpt * T;
+    int c = 32;
+    while (c < need) c <<= 1;
+    return c;
+}
+
 // Floats per vehicle of a stored state (checkpoints, sub-checkpoints, the
 // adjoint's state stage): position high and low parts, speed, raw gap and the
 // compensation of the speed sum (State2).
@@ -106,7 +121,7 @@ cudaError_t launch_forward(int vpt, int G, bool traj, bool vtraj, bool ckpt, con
                            cudaStream_t st);
 cudaError_t launch_backward(int vpt, int G, bool dense_seed, bool adam, bool want_delta, const SimArgs &a,
                             int grid, int wpb, cudaStream_t st);
-size_t backward_smem_bytes(int vpt, bool dense_seed, int T, int G, int wpb, bool prefetch);
+size_t backward_smem_bytes(int vpt, int T, int G, int wpb, bool prefetch);
 size_t forward_smem_bytes(int vpt, int G, int wpb);
 // Largest adjoint block (warps) for a shape: 4 for 4 vehicles per thread in
 // segments of up to 4 warps (register budget), else 8.
@@ -130,8 +145,11 @@ cudaError_t launch_fit_fused(int vpt, int G, const SimArgs &a, long long part_st
 // each summed in the order of launch_loss_finalize.
 cudaError_t launch_loss_finalize_iters(const double *loss_part, long long stride, const int *n_seg, int per_seg,
                                        int n_iter, double *out, cudaStream_t st);
-int occupancy_blocks(int vpt, int G, bool backward, bool dense_seed, bool adam, bool want_delta, int wpb, size_t smem,
-                     bool sub = false);
+// Resident blocks per SM (at least 1) of the forward, and of the adjoint with
+// `cols` tensor-memory columns per block.
+int forward_blocks_per_sm(int vpt, int G, int wpb);
+int backward_blocks_per_sm(int vpt, int G, bool dense_seed, bool adam, bool want_delta, int wpb, size_t smem, bool sub,
+                           int cols);
 // Kernel shapes (vehicles per thread, warps per segment) with compiled
 // adjoint and single-launch fit kernels; X(V, G) per shape.
 #define IDM_SHAPES(X) \
@@ -139,11 +157,11 @@ int occupancy_blocks(int vpt, int G, bool backward, bool dense_seed, bool adam, 
 // Per shape (idm_shape_v<V>_g<G>.cu): the forward kernel (with or without
 // event counting), the adjoint kernel for dense or target seeds, fused Adam,
 // the delta gradient and tape blocks with sub-checkpoints, and the
-// single-launch fit kernel (tape blocks or not).
+// single-launch fit kernel (tape blocks or not); consec: the slot mapping.
 #define IDM_DECLARE_SHAPE(V, GW)                                             \
     void *forward_fn_v##V##_g##GW(bool count);                                \
-    void *backward_fn_v##V##_g##GW(bool dense, bool adam, bool wd, bool sub); \
-    void *fused_fn_v##V##_g##GW(bool sub);
+    void *backward_fn_v##V##_g##GW(bool dense, bool adam, bool wd, bool sub, bool consec); \
+    void *fused_fn_v##V##_g##GW(bool sub, bool consec);
 IDM_SHAPES(IDM_DECLARE_SHAPE)
 #undef IDM_DECLARE_SHAPE
 

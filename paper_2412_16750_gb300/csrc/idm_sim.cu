@@ -335,9 +335,9 @@ cudaError_t launch_forward(int vpt, int G, bool traj, bool vtraj, bool ckpt, con
     return cudaLaunchKernel(fn, dim3(grid), dim3(32 * wpb), params, smem, st);
 }
 
-size_t backward_smem_bytes(int vpt, bool dense_seed, int T, int G, int wpb, bool prefetch)
+size_t backward_smem_bytes(int vpt, int T, int G, int wpb, bool prefetch)
 {
-    return (size_t)bwd_group_floats(vpt, dense_seed, T, G, prefetch) * (wpb / G) * sizeof(float);
+    return (size_t)bwd_group_floats(vpt, T, G, prefetch) * (wpb / G) * sizeof(float);
 }
 
 size_t forward_smem_bytes(int vpt, int G, int wpb)
@@ -346,17 +346,51 @@ size_t forward_smem_bytes(int vpt, int G, int wpb)
     return (size_t)grp_ctrl_floats(G) * (wpb / G) * sizeof(float);
 }
 
+// The slot mapping of a fit's adjoint: a scene's vehicles four to a thread in a
+// row (2M x 1,000 at interval 50: 15.45 -> 15.22 ms per iteration); a batch's
+// interleaved, because its losses are reported per scenario, and a scenario's
+// FP32 partial sums by thread keep their grouping.  Loss and gradient without
+// Adam stay interleaved too (10,000 lanes of 2-200 vehicles, 301 steps: 2.23 ms
+// against 2.31).
+static bool consecutive_slots(const SimArgs &a) { return a.scen_tab == nullptr; }
+
 // Adjoint variants of every shape live in idm_shape_v<V>_g<G>.cu (with
 // 4 vehicles per thread, segments of up to 4 warps run in 4-warp blocks and
 // 8-warp segments in 8-warp blocks); SUB: tape shallower than the checkpoint
 // interval.
-static void *backward_fn_v(int vpt, int G, bool dense, bool adam, bool wd, bool sub)
+static void *backward_fn_v(int vpt, int G, bool dense, bool adam, bool wd, bool sub, bool consec)
 {
 #define IDM_PICK(V, GW) \
-    if (vpt == V && G == GW) return backward_fn_v##V##_g##GW(dense, adam, wd, sub);
+    if (vpt == V && G == GW) return backward_fn_v##V##_g##GW(dense, adam, wd, sub, consec);
     IDM_SHAPES(IDM_PICK)
 #undef IDM_PICK
     return nullptr;
+}
+
+// Resident blocks per SM of a kernel that allocates `cols` tensor-memory
+// columns per block, from its registers, shared memory and columns (the
+// runtime's occupancy query answers 1 for any kernel that allocates tensor
+// memory).  A block waits for its columns, so no more than fit are launched.
+static int adjoint_blocks_per_sm(const void *fn, int G, int wpb, size_t smem, int cols)
+{
+    cudaFuncAttributes at;
+    if (cudaFuncGetAttributes(&at, fn) != cudaSuccess) return 1;
+    const int regs = (at.numRegs + 7) / 8 * 8 * 32 * wpb;
+    const size_t sh = (smem + at.sharedSizeBytes + 127) / 128 * 128 + 1024;
+    int n = 65536 / regs;
+    n = n < (int)(228 * 1024 / sh) ? n : (int)(228 * 1024 / sh);
+    n = n < TMEM_COLS / cols ? n : TMEM_COLS / cols;
+    // 64 named barriers per SM, 16 per block where groups have them (their ids are run-time values)
+    if (G > 1) n = n < 4 ? n : 4;
+    n = n < 64 / wpb ? n : 64 / wpb;
+    n = n < 32 ? n : 32;
+    return n > 1 ? n : 1;
+}
+
+int backward_blocks_per_sm(int vpt, int G, bool dense, bool adam, bool want_delta, int wpb, size_t smem, bool sub, int cols)
+{
+    void *fn = backward_fn_v(vpt, G, dense, adam, want_delta && !adam, sub, true);
+    return fn ? adjoint_blocks_per_sm(fn, G, wpb, smem, cols) : 1;
 }
 
 int backward_max_warps(int vpt, int G) { return (vpt == 4 && G <= 4) ? 4 : 8; }
@@ -372,10 +406,10 @@ cudaError_t launch_backward(int vpt, int G, bool dense_seed, bool adam, bool wan
                             int wpb, cudaStream_t st)
 {
     if (dense_seed && adam) return cudaErrorInvalidValue;
-    if (wpb > backward_max_warps(vpt, G) || wpb % G) return cudaErrorInvalidValue;
-    void *fn = backward_fn_v(vpt, G, dense_seed, adam, want_delta && !adam, a.tape_T < a.C);
+    if (wpb > backward_max_warps(vpt, G) || wpb % G || a.tape_cols > TMEM_COLS) return cudaErrorInvalidValue;
+    void *fn = backward_fn_v(vpt, G, dense_seed, adam, want_delta && !adam, a.tape_T < a.C, consecutive_slots(a));
     if (!fn) return cudaErrorInvalidValue;
-    size_t smem = backward_smem_bytes(vpt, dense_seed, a.tape_T, G, wpb, a.bwd_pf != 0);
+    size_t smem = backward_smem_bytes(vpt, a.tape_T, G, wpb, a.bwd_pf != 0);
     cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     SimArgs args = a;
@@ -385,10 +419,10 @@ cudaError_t launch_backward(int vpt, int G, bool dense_seed, bool adam, bool wan
 }
 
 // Single-launch fit kernels of every shape live in idm_shape_v<V>_g<G>.cu.
-static void *fused_fn_v(int vpt, int G, bool sub)
+static void *fused_fn_v(int vpt, int G, bool sub, bool consec)
 {
 #define IDM_PICK(V, GW) \
-    if (vpt == V && G == GW) return fused_fn_v##V##_g##GW(sub);
+    if (vpt == V && G == GW) return fused_fn_v##V##_g##GW(sub, consec);
     IDM_SHAPES(IDM_PICK)
 #undef IDM_PICK
     return nullptr;
@@ -397,19 +431,16 @@ static void *fused_fn_v(int vpt, int G, bool sub)
 cudaError_t launch_fit_fused(int vpt, int G, const SimArgs &a, long long part_stride, int grid, int wpb,
                              cudaStream_t st)
 {
-    if (wpb > backward_max_warps(vpt, G) || wpb % G) return cudaErrorInvalidValue;
-    void *fn = fused_fn_v(vpt, G, a.tape_T < a.C);
+    if (wpb > backward_max_warps(vpt, G) || wpb % G || a.tape_cols > TMEM_COLS) return cudaErrorInvalidValue;
+    void *fn = fused_fn_v(vpt, G, a.tape_T < a.C, consecutive_slots(a));
     if (!fn) return cudaErrorInvalidValue;
-    const size_t smem = backward_smem_bytes(vpt, false, a.tape_T, G, wpb, a.bwd_pf != 0);
+    const size_t smem = backward_smem_bytes(vpt, a.tape_T, G, wpb, a.bwd_pf != 0);
     cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    int occ = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, 32 * wpb, smem);
     if (e != cudaSuccess) return e;
     int dev = 0, n_sm = 1;
     if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
     if ((e = cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-    const int cap = n_sm * (occ > 0 ? occ : 1);
+    const int cap = n_sm * adjoint_blocks_per_sm(fn, G, wpb, smem, a.tape_cols);
     SimArgs args = a;
     args.G = G;
     long long stride = part_stride;
@@ -417,19 +448,12 @@ cudaError_t launch_fit_fused(int vpt, int G, const SimArgs &a, long long part_st
     return cudaLaunchKernel(fn, dim3(grid < cap ? grid : cap), dim3(32 * wpb), params, smem, st);
 }
 
-int occupancy_blocks(int vpt, int G, bool backward, bool dense, bool adam, bool want_delta, int wpb, size_t smem,
-                     bool sub)
+int forward_blocks_per_sm(int vpt, int G, int wpb)
 {
-    void *fn = nullptr;
-    if (!backward) {
-        fn = forward_fn_v(vpt, G, false);
-        smem = forward_smem_bytes(vpt, G, wpb);
-        if (fn) cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    } else {
-        fn = backward_fn_v(vpt, G, dense, adam, want_delta && !adam, sub);
-        if (fn) cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    }
+    void *fn = forward_fn_v(vpt, G, false);
     if (!fn) return 1;
+    const size_t smem = forward_smem_bytes(vpt, G, wpb);
+    cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     int n = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, fn, 32 * wpb, smem) != cudaSuccess) return 1;
     return n > 0 ? n : 1;

@@ -48,17 +48,34 @@ __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commi
 template <int N>
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
-// Slots of a warp: pair p of lane l holds slots 64p + 2l and 64p + 2l + 1.
-// dst/src_row already point at this warp's first slot.
-template <int NP>
-__device__ __forceinline__ void prefetch_row(float *dst, const float *src_row, int lane, const bool (&vx)[NP],
-                                             const bool (&vy)[NP])
+__device__ __forceinline__ void cp_async16(float *smem_dst, const float *gsrc)
 {
+    unsigned s = (unsigned)__cvta_generic_to_shared(smem_dst);
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(s), "l"(gsrc) : "memory");
+}
+
+// Offset of pair p from the lane's first slot.
+template <bool CONSEC>
+__device__ __forceinline__ constexpr int pair_off(int p)
+{
+    return CONSEC ? 2 * p : 64 * p;
+}
+
+// Copy this lane's occupied slots (mask) of one row: dst and src point at the
+// lane's first slot.  vec: all 2 NP slots are occupied and consecutive and the
+// source is 16-byte aligned.
+template <int NP, bool CONSEC>
+__device__ __forceinline__ void prefetch_row(float *dst, const float *src, const int (&mask)[NP][2], bool vec)
+{
+    if (CONSEC && NP >= 2 && vec) {
 #pragma unroll
-    for (int p = 0; p < NP; ++p) {
-        const int q = 64 * p + 2 * lane;
-        if (vx[p]) cp_async4(dst + q, src_row + q);
-        if (vy[p]) cp_async4(dst + q + 1, src_row + q + 1);
+        for (int c = 0; c < 2 * NP; c += 4) cp_async16(dst + c, src + c);
+    } else {
+#pragma unroll
+        for (int p = 0; p < NP; ++p)
+#pragma unroll
+            for (int c = 0; c < 2; ++c)
+                if (mask[p][c]) cp_async4(dst + pair_off<CONSEC>(p) + c, src + pair_off<CONSEC>(p) + c);
     }
 }
 
@@ -76,12 +93,15 @@ struct Grp {
     int lane;
     int bar;     // named barrier id (1 + group index in the block)
     int *cell;   // [2] work-item broadcast
-    float *xl;   // [2][G][2] leader exchange (speed, speed compensation)
-    float *xf;   // [2][2][G] follower exchange
+    // exchange cells, double-buffered by parity (xp, fp: 0 or G + 1): warp w
+    // writes its last slot's speed and compensation to cell w + 1 of xl and
+    // reads cell w; writes its first slot's follower terms to cell w of xf and
+    // reads cell w + 1.  Cells 0 of xl and G of xf stay 0 (no neighbour).
+    float2 *xl, *xf;
 };
 
 // Shared floats of one group's control area (cells + exchange cells).
-__host__ __device__ __forceinline__ int grp_ctrl_floats(int G) { return ((2 + 8 * G) + 3) & ~3; }
+__host__ __device__ __forceinline__ int grp_ctrl_floats(int G) { return (2 + 8 * (G + 1) + 3) & ~3; }
 
 __device__ __forceinline__ void grp_sync(const Grp &g)
 {
@@ -100,8 +120,13 @@ __device__ __forceinline__ Grp make_grp(int G, float *ctrl)
     g.lane = threadIdx.x & 31;
     g.bar = 1 + warp / G;
     g.cell = reinterpret_cast<int *>(ctrl);
-    g.xl = ctrl + 2;
-    g.xf = ctrl + 2 + 4 * G;
+    g.xl = reinterpret_cast<float2 *>(ctrl + 2);
+    g.xf = g.xl + 2 * (G + 1);
+    if (G > 1 && g.lane < 2) {  // every warp writes the zeros that it may read
+        g.xl[g.lane * (G + 1)] = make_float2(0.0f, 0.0f);
+        g.xf[g.lane * (G + 1) + G] = make_float2(0.0f, 0.0f);
+    }
+    __syncwarp();
     return g;
 }
 
@@ -121,58 +146,58 @@ __device__ __forceinline__ int grp_next(const Grp &g, int *work, int &par)
 __device__ __forceinline__ float2 grp_lead_in(const Grp &g, float2 last, int &xp)
 {
     if (g.G == 1) return make_float2(0.0f, 0.0f);
-    float2 *c = reinterpret_cast<float2 *>(g.xl);
-    if (g.lane == 31) c[xp * g.G + g.w] = last;
+    float2 *c = g.xl + xp + g.w;
+    if (g.lane == 31) c[1] = last;
     grp_sync(g);
-    const float2 r = g.w > 0 ? c[xp * g.G + g.w - 1] : make_float2(0.0f, 0.0f);
-    xp ^= 1;
-    return r;
+    xp = g.G + 1 - xp;
+    return c[0];
 }
 
-// Follower terms arriving at this warp's last slot (0 for the last warp).
-__device__ __forceinline__ void grp_follow_in(const Grp &g, float p_first, float v_first, float &in_p, float &in_v,
-                                              int &xp)
+// Follower terms (of position and speed) arriving at this warp's last slot (0
+// for the last warp); first: this lane's of the warp's first slot (used by
+// lane 0).
+__device__ __forceinline__ float2 grp_follow_in(const Grp &g, float2 first, int &fp)
 {
-    in_p = 0.0f;
-    in_v = 0.0f;
-    if (g.G == 1) return;
-    float *c = g.xf + xp * 2 * g.G;
-    if (g.lane == 0) {
-        c[g.w] = p_first;
-        c[g.G + g.w] = v_first;
-    }
+    if (g.G == 1) return make_float2(0.0f, 0.0f);
+    float2 *c = g.xf + fp + g.w;
+    if (g.lane == 0) c[0] = first;
     grp_sync(g);
-    if (g.w + 1 < g.G) {
-        in_p = c[g.w + 1];
-        in_v = c[g.G + g.w + 1];
-    }
-    xp ^= 1;
+    fp = g.G + 1 - fp;
+    return c[1];
 }
 
-// One Euler step (Eq. 1-3 with the Sec. III-C bounds) of this thread's
-// vehicle pairs: the leaders' speeds and speed compensations by shuffle
-// (across warps through the group's cells), then a* and the state update.
-template <int NP, bool D4>
-__device__ __forceinline__ void step_pairs(const Grp &g, State2 (&st)[NP], const VehConst2 (&kc)[NP],
-                                           const ScenDesc &sc, int &xp)
+// Speed and compensation differences to the leaders (by shuffle; across warps
+// through the group's cells).
+template <int NP, bool CONSEC>
+__device__ __forceinline__ void leader_diffs(const Grp &g, const State2 (&st)[NP], f2 (&dv)[NP], f2 (&dvc)[NP], int &xp)
 {
-    f2 vcur[NP], ccur[NP], vh[NP], ch[NP];
+    f2 vcur[NP], ccur[NP];
 #pragma unroll
     for (int p = 0; p < NP; ++p) {
         vcur[p] = st[p].v;
         ccur[p] = st[p].vc;
     }
     const float2 lead_in = grp_lead_in(g, make_float2(vcur[NP - 1].y, ccur[NP - 1].y), xp);
-    leader_vals2<NP>(vcur, vh, g.lane, lead_in.x);
-    leader_vals2<NP>(ccur, ch, g.lane, lead_in.y);
+    minus_leader2<NP, CONSEC>(vcur, dv, g.lane, lead_in.x);
+    minus_leader2<NP, CONSEC>(ccur, dvc, g.lane, lead_in.y);
+}
+
+// One Euler step (Eq. 1-3 with the Sec. III-C bounds) of this thread's
+// vehicle pairs.
+template <int NP, bool D4, bool CONSEC>
+__device__ __forceinline__ void step_pairs(const Grp &g, State2 (&st)[NP], const VehConst2 (&kc)[NP],
+                                           const ScenDesc &sc, int &xp)
+{
+    f2 dv[NP], dvc[NP];
+    leader_diffs<NP, CONSEC>(g, st, dv, dvc, xp);
 #pragma unroll
     for (int p = 0; p < NP; ++p) {
-        const f2 as = accel_star2<D4>(st[p].v, st[p].gap, vh[p], kc[p], sc.inv_dt, sc.a_min);
-        euler2(st[p], as, vh[p], ch[p], sc.dt);
+        const f2 as = accel_star2<D4>(st[p].v, st[p].gap, dv[p], kc[p], sc.inv_dt, sc.a_min);
+        euler2(st[p], as, dv[p], dvc[p], sc.dt);
     }
 }
 
-template <int NP>
+template <int NP, bool CONSEC>
 __device__ __forceinline__ void load_vehicles(const SimArgs &a, const Seg &sg, int lane, int wb, VehConst2 (&kc)[NP],
                                               State2 (&st)[NP], bool (&vx)[NP], bool (&vy)[NP])
 {
@@ -180,7 +205,7 @@ __device__ __forceinline__ void load_vehicles(const SimArgs &a, const Seg &sg, i
     for (int p = 0; p < NP; ++p) {
 #pragma unroll
         for (int c = 0; c < 2; ++c) {
-            const int q = wb + 64 * p + 2 * lane + c;
+            const int q = wb + pair_slot<NP, CONSEC>(p, lane) + c;
             const bool ok = q < sg.n_veh;
             float inv_v0 = 1.0f, T = 0.0f, s0 = 0.0f, am = 1.0f, cc = 0.5f, dl = 4.0f;  // ghost slot
             float ph = 0.0f, v = 0.0f, gap = INFINITY;
@@ -240,19 +265,51 @@ __device__ __forceinline__ f2 load_pair(const float *base, int q, bool vx, bool 
 }
 
 
-__device__ __forceinline__ f2 lds2(const float *p) { return *reinterpret_cast<const f2 *>(p); }
-__device__ __forceinline__ void sts2(float *p, f2 x) { *reinterpret_cast<f2 *>(p) = x; }
-
-// Shared floats of one adjoint group: tape v/gap [T][G*SL], target/seed
-// tapes [T][G*SL] (MSE only), state stages [STATE_ROWS][G*SL], control area; T is the tape depth (the checkpoint interval, or less when
-// blocks restart from sub-checkpoints).  With prefetch the target tape and
-// the state stage are doubled and the next block's targets and starting
-// state are copied (cp.async) into the idle pair while the current block
-// runs.
-__host__ __device__ __forceinline__ int bwd_group_floats(int vpt, bool dense, int T, int G, bool pf)
+// This lane's pairs of a shared row (consecutive ones 16 bytes at a time).
+template <int NP, bool CONSEC>
+__device__ __forceinline__ void lds_row(const float *r, f2 (&x)[NP])
 {
-    const int nb = pf ? 2 : 1;
-    return ((dense ? 2 : 2 + nb) * T + STATE_ROWS * nb) * 32 * vpt * G + grp_ctrl_floats(G);
+    if (NP == 1 || !CONSEC) {
+#pragma unroll
+        for (int p = 0; p < NP; ++p) x[p] = *reinterpret_cast<const f2 *>(r + pair_off<CONSEC>(p));
+    } else {
+#pragma unroll
+        for (int p = 0; p + 1 < NP; p += 2) {
+            const float4 v = *reinterpret_cast<const float4 *>(r + 2 * p);
+            x[p] = make_float2(v.x, v.y);
+            x[p + 1] = make_float2(v.z, v.w);
+        }
+    }
+}
+template <int NP, bool CONSEC>
+__device__ __forceinline__ void sts_row(float *r, const f2 (&x)[NP])
+{
+    if (NP == 1 || !CONSEC) {
+#pragma unroll
+        for (int p = 0; p < NP; ++p) *reinterpret_cast<f2 *>(r + pair_off<CONSEC>(p)) = x[p];
+    } else {
+#pragma unroll
+        for (int p = 0; p + 1 < NP; p += 2)
+            *reinterpret_cast<float4 *>(r + 2 * p) = make_float4(x[p].x, x[p].y, x[p + 1].x, x[p + 1].y);
+    }
+}
+
+// Shared floats of one adjoint group: tapes of speeds, frd and targets (dense
+// seeds) turned seeds, [T][G*SL] each, a state stage [STATE_ROWS][G*SL] laid
+// over the first two (the targets start at row bwd_target_row), and the control
+// area; T is the tape depth (the checkpoint interval, or less when
+// blocks restart from sub-checkpoints).  With prefetch the target tape is
+// doubled and the state stage apart, and the next block's rows and starting
+// state are copied (cp.async) while the current block runs (the state stage is
+// free as soon as the block has loaded its own).
+__host__ __device__ __forceinline__ int bwd_target_row(int T, bool pf)
+{
+    return pf || 2 * T > STATE_ROWS ? 2 * T : STATE_ROWS;
+}
+__host__ __device__ __forceinline__ int bwd_group_floats(int vpt, int T, int G, bool pf)
+{
+    const int rows = bwd_target_row(T, pf) + (pf ? 2 * T + STATE_ROWS : T);
+    return rows * 32 * vpt * G + grp_ctrl_floats(G);
 }
 
 }  // namespace idm

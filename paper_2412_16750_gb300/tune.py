@@ -4,7 +4,7 @@ A shape is (vpt, warps_per_segment, ckpt_interval, warps_per_block) as taken
 by idm_set_tuning: vehicles per thread and warps per lane segment fix the
 segment capacity 32 * vpt * warps (lanes are packed into segments of that
 size), the checkpoint interval sets the adjoint's recompute length and
-shared-memory tape, and warps per block the persistent grid.  The best shape
+tape, and warps per block the persistent grid.  The best shape
 depends on the lane-length mix, the horizon and the GPU, so it is measured:
 the caller supplies one run of its workload (a loss + gradient or a fit
 iteration), the tuner times it for candidate shapes with CUDA events and
