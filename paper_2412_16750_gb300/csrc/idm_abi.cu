@@ -201,7 +201,15 @@ static int prepare(idm_ctx *c, const idm_scene_t *sc, const idm_params_t *pr, co
     if ((rc = ensure(c, c->loss_tmp, sizeof(double) * 2, "loss scalar"))) return rc;
     // an interval longer than the horizon gives the same single checkpoint
     // segment; clamping it lets the adjoint's tape be only K steps deep
-    const int C = std::min(c->C, sim->K);
+    int C = std::min(c->C, sim->K), split = 0;
+    // a horizon of up to two intervals that the tape of 2 vehicles per thread
+    // holds whole (16 steps) is one segment too: a fit's forward then runs once
+    // (the one checkpoint is the initial state); the loss keeps the sums of the
+    // interval's segments
+    if (P->vpt == 2 && sim->K > C && sim->K <= 2 * C && sim->K <= 16) {
+        split = C;
+        C = sim->K;
+    }
     const int n_ck = (sim->K + C - 1) / C;
     if (need_ckpt &&
         (rc = ensure(c, c->ckpt, sizeof(float) * idm::STATE_ROWS * (size_t)n_ck * N, "checkpoints")))
@@ -230,6 +238,7 @@ static int prepare(idm_ctx *c, const idm_scene_t *sc, const idm_params_t *pr, co
     a.loss_part = (double *)c->loss_part.p;
     a.ckpt = (float *)c->ckpt.p;
     a.C = C;
+    a.loss_split = split;
     a.status = (unsigned *)c->status.p;
     a.N_total = N;
     a.G = G;
