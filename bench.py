@@ -673,9 +673,9 @@ def batched(a, dev):
 
 # Algorithmic bytes per trajectory-step of one fit iteration of the
 # reconstruction mode: forward reads dp, dv and the observation row (16 B)
-# and writes the tape (32 B); the adjoint reads the tape, dp, dv and four Adam
-# moments (56 B) and writes dp, dv and the moments (24 B).
-RECON_BYTES_PER_STEP = 16 + 32 + 56 + 24
+# and writes speed and seed (8 B); the adjoint reads them, dp, dv and four Adam
+# moments (32 B) and writes dp, dv and the moments (24 B).
+RECON_BYTES_PER_STEP = 16 + 8 + 32 + 24
 
 
 def reconstruction(a, dev):
@@ -1066,7 +1066,7 @@ def run_gpu(a, rank, world, local_rank):
                  "ms_per_step": mt["ms"] / a.tuned_steps,
                  "fwd_ms_per_timestep": mt["fwd_avg_ms"] / K, "bwd_ms_per_timestep": mt["bwd_avg_ms"] / K,
                  "roofline": adjoint_roofline(N, K, a.tuned_ckpt, mt["bwd_avg_ms"], n_sm, peaks, peak_kind),
-                 "note": "the same workload with the checkpoint interval whose adjoint tape fits shared memory "
+                 "note": "the same workload with the checkpoint interval whose adjoint tape fits the chip "
                          "(no tape blocks); checkpoints then take %.1f GB instead of %.2f GB"
                          % (16.0 * N * math.ceil(K / a.tuned_ckpt) / 1e9, 16.0 * N * math.ceil(K / a.ckpt) / 1e9)}
         ctx.set_tuning(a.vpt, a.G, a.ckpt, a.wpb)

@@ -583,7 +583,8 @@ __device__ __forceinline__ void backward_segment_blocks(const SimArgs &a, const 
     // Block j > 0 of a checkpoint segment starts from sub-checkpoint row j - 1,
     // block 0 from the checkpoint.  With several vehicle pairs per thread (tapes
     // of 8 steps) the first block takes the remainder: the forward pass then
-    // ends where the last full block begins (42 steps of 50 instead of 48).
+    // ends where the last full block begins (42 steps of 50 instead of 48: two
+    // iterations of 2M x 1,000 31.13 -> 30.89 ms).
     constexpr bool SHORT_FIRST = NP >= 2;
     auto seg_len = [&](int cs) { return min(a.C, sc.K - cs * a.C); };
     auto n_sub = [&](int cs) { return (seg_len(cs) + T - 1) / T; };
