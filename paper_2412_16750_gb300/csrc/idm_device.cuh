@@ -350,17 +350,20 @@ __device__ __forceinline__ f2 accel_jac2(f2 v, f2 gap_raw, f2 dv, const VehConst
     return add2(a_lb, s2.sp);
 }
 
-// sigma2 r^delta ln r of a step from its speed and frd = sigma2 r^delta.
-// r^delta ln r -> 0 as r -> 0+.  Near rest the a_lb = -v/dt branch leaves v +
-// dt a* within rounding of 0: a speed a few ulps below 0, or a denormal that
-// the flush-to-zero logarithm reads as 0, take the limit too: r^delta has
-// (all but) underflowed there, and with D4 the logarithm's argument is held
-// above 1e-37, so that the product is 0 to 1e-20.
+// sigma2 r^delta ln r of a step from its speed and frd = sigma2 r^delta, 0 for
+// r <= 0: the limit r -> 0+ near rest (where the a_lb = -v/dt branch leaves v +
+// dt a* within rounding of 0), and the value taken at a caller's negative
+// initial speed, whose r^4 is not small.  With D4 the logarithm's argument is
+// held above 1e-37, so that a denormal speed, which the flush-to-zero logarithm
+// reads as 0, gives 0 * finite.
 template <bool D4>
 __device__ __forceinline__ f2 delta_factor2(f2 v, f2 frd, const VehConst2 &k)
 {
     const f2 r = mul2(v, k.inv_v0);
-    if (D4) return mul2(frd, mul2(lg2(vmax(r, F2(1e-37f))), F2(LN2)));
+    if (D4) {
+        const f2 t = mul2(frd, mul2(lg2(vmax(r, F2(1e-37f))), F2(LN2)));
+        return make_float2(r.x > 0.0f ? t.x : 0.0f, r.y > 0.0f ? t.y : 0.0f);
+    }
     const f2 rd = pow_delta2<D4>(r, k.delta);
     const f2 t = mul2(frd, mul2(lg2(r), F2(LN2)));
     return make_float2(r.x > 0.0f && rd.x > 0.0f ? t.x : 0.0f, r.y > 0.0f && rd.y > 0.0f ? t.y : 0.0f);
