@@ -112,8 +112,6 @@ constexpr int STATE_ROWS = 5;
 // Launchers (idm_sim.cu).  Return cudaError_t of the launch.
 cudaError_t launch_prep_gap(const int *lane_off, int n_lanes, const float *p_init, const float *length,
                             int N, float *g0, unsigned *status, cudaStream_t st);
-cudaError_t launch_build_segments(const int *lane_off, int n_lanes, int cap, int N, bool one_wave, Seg *seg, int *n_seg,
-                                  unsigned *status, cudaStream_t st);
 // The kernel shape (vehicles per thread, warps per segment) of each launch is
 // passed explicitly; the forward and the adjoint may differ as long as
 // 32 * vpt * G (the segment capacity the segments were packed for) agrees.
