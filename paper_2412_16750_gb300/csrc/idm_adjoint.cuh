@@ -1,6 +1,8 @@
 // Adjoint kernel templates; each idm_shape_v<VPT>_g<G>.cu instantiates the
 // variants of one kernel shape (so they compile in parallel).
 #pragma once
+#include <limits.h>
+
 #include "idm_gemm_tc.cuh"
 #include "idm_sim_common.cuh"
 
@@ -43,6 +45,15 @@ namespace idm {
 // pair, each written and read back by the thread that owns the pair.
 // ---------------------------------------------------------------------------
 constexpr int FOLD_STEPS = GSUM_FOLD_STEPS;
+
+// Checkpoint segments per fold.  Without totals the sums stay in registers: a
+// call whose horizons are within FOLD_STEPS has none, although such a horizon can
+// have more segments than a window (251-256 steps at interval 50: six of them,
+// five to a window).
+__device__ __forceinline__ int folds_every(const SimArgs &a)
+{
+    return a.gsum ? max(1, FOLD_STEPS / a.C) : INT_MAX;
+}
 
 // ---------------------------------------------------------------------------
 // The tape's tensor-memory part: per step TAPE_WORDS * VPT 32-bit columns of
@@ -547,7 +558,7 @@ __device__ __forceinline__ void backward_segment(const SimArgs &a, const ScenDes
                    a.ckpt + sc.ckpt_off + (size_t)cs * STATE_ROWS * sc.n_veh + w.wl, (size_t)sc.n_veh);
     };
     const int n_ck = (sc.K + a.C - 1) / a.C;
-    const int fold_every = max(1, FOLD_STEPS / a.C);  // checkpoint segments per fold of the gradient sums
+    const int fold_every = folds_every(a);
     if (nb > 1) prefetch(n_ck - 1);
     for (int cs = n_ck - 1; cs >= 0; --cs) {
         const int par = nb > 1 ? cs & 1 : 0, c0 = cs * a.C;
@@ -598,7 +609,7 @@ __device__ __forceinline__ void backward_segment_blocks(const SimArgs &a, const 
                    j == 0 ? ckpt_row(cs) : sub_row(j), j == 0 ? (size_t)sc.n_veh : (size_t)a.N_total);
     };
     const int n_ck = (sc.K + a.C - 1) / a.C;
-    const int fold_every = max(1, FOLD_STEPS / a.C);
+    const int fold_every = folds_every(a);
     int par = 0;
     bool have_next = false;  // the next block's stage is already being filled
     if (nb > 1 && n_sub(n_ck - 1) == 1) {

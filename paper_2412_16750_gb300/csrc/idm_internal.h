@@ -76,8 +76,8 @@ struct SimArgs {
     // (needs more shared memory), 0 = load each segment when it starts
     int bwd_pf;
     // adjoint: compensated running totals of the six factored gradient sums,
-    // per segment 6 x (capacity / 2) float4 (16-byte aligned); needed
-    // (non-NULL) when a horizon exceeds GSUM_FOLD_STEPS
+    // per segment 6 x (capacity / 2) float4 (16-byte aligned); needed when a
+    // horizon exceeds GSUM_FOLD_STEPS, else NULL and the sums are not folded
     float *gsum;
     // forward: event counters (NULL = not counted): [0] vehicle-steps with the
     // raw gap below the floor, [1] vehicle-steps within IDM_KINK_BAND of the
