@@ -340,12 +340,13 @@ int backward_grid(idm_ctx *c, Prep *P, bool dense, bool adam, bool want_delta, i
     P->a.bwd_pf = pf ? 1 : 0;
     P->a.tape_T = T;
     // compensated totals of the gradient sums (folded only past the window),
-    // for the most segments the packing can produce (L: lanes of a single
-    // scene, or the batch's segments)
+    // for the batch's segments (L), or the most that the packing of a scene's L
+    // lanes can produce
     if (P->k_max > idm::GSUM_FOLD_STEPS && P->a.N_total > 0) {
         const long long cap = 32LL * P->vpt * G;
-        const long long n_seg = std::min<long long>(
-            L, 2 * (((long long)P->a.N_total + cap - 1) / cap) + idm::SEG_BUILD_CHUNKS);
+        const long long n_seg =
+            P->a.scen_tab ? L
+                          : std::min<long long>(L, 2 * (((long long)P->a.N_total + cap - 1) / cap) + idm::SEG_BUILD_CHUNKS);
         int rc;
         if ((rc = ensure(c, c->gsum, idm::gsum_bytes((size_t)n_seg, (int)cap), "gradient totals"))) return rc;
         P->a.gsum = (float *)c->gsum.p;
