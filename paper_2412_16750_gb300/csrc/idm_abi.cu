@@ -344,9 +344,7 @@ int backward_grid(idm_ctx *c, Prep *P, bool dense, bool adam, bool want_delta, i
     // lanes can produce
     if (P->k_max > idm::GSUM_FOLD_STEPS && P->a.N_total > 0) {
         const long long cap = 32LL * P->vpt * G;
-        const long long n_seg =
-            P->a.scen_tab ? L
-                          : std::min<long long>(L, 2 * (((long long)P->a.N_total + cap - 1) / cap) + idm::SEG_BUILD_CHUNKS);
+        const long long n_seg = P->a.scen_tab ? L : idm::segment_bound(P->a.N_total, L, cap);
         int rc;
         if ((rc = ensure(c, c->gsum, idm::gsum_bytes((size_t)n_seg, (int)cap), "gradient totals"))) return rc;
         P->a.gsum = (float *)c->gsum.p;
@@ -483,10 +481,7 @@ int run_fit_graph(idm_ctx *c, Prep &P, int n_iter, size_t N, const float *box_lo
 // most segments the packing can produce (see run_fit_single).
 long long single_launch_stride(const Prep &P, size_t N, int n_lanes)
 {
-    const long long cap = 32LL * P.vpt * P.G;
-    const long long seg_bound =
-        std::min<long long>(n_lanes, 2 * (((long long)N + cap - 1) / cap) + idm::SEG_BUILD_CHUNKS);
-    return std::max<long long>(1, seg_bound * P.G);
+    return std::max<long long>(1, idm::segment_bound((long long)N, n_lanes, 32LL * P.vpt * P.G) * P.G);
 }
 
 // The fit as one persistent launch (idm_fused.cuh) for a single scene:

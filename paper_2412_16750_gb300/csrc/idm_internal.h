@@ -27,6 +27,11 @@ struct ScenDesc {
 // thread each, next-fit inside a chunk), so n vehicles in lanes no longer
 // than the capacity give at most 2 n / cap + SEG_BUILD_CHUNKS segments.
 constexpr int SEG_BUILD_CHUNKS = 1024;
+__host__ __device__ inline long long segment_bound(long long n_vehicles, long long n_lanes, long long cap)
+{
+    const long long b = 2 * ((n_vehicles + cap - 1) / cap) + SEG_BUILD_CHUNKS;
+    return n_lanes < b ? n_lanes : b;
+}
 
 // One warp segment: whole lanes packed into at most 32*VPT slots.
 struct Seg {

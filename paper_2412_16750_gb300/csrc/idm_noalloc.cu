@@ -134,10 +134,7 @@ extern "C" int idm_loss_grad_noalloc(const idm_scene_t *sc, const idm_params_t *
     const bool totals = sim->K > idm::GSUM_FOLD_STEPS && N > 0;
     const long long cap = 32LL * P.vpt * G;
     const size_t totals_bytes =
-        totals ? idm::gsum_bytes((size_t)std::min<long long>((long long)L, 2 * (((long long)N + cap - 1) / cap) +
-                                                                               idm::SEG_BUILD_CHUNKS),
-                                 (int)cap)
-               : 0;
+        totals ? idm::gsum_bytes((size_t)idm::segment_bound((long long)N, (long long)L, cap), (int)cap) : 0;
 
     // scratch layout (256-byte aligned pieces)
     size_t off = 0;

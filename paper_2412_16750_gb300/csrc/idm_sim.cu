@@ -195,7 +195,9 @@ __device__ __forceinline__ void build_segments(const int *lane_off, int n_lanes,
     } else {
         pack_lanes<true>(lane_off, l0, l1, cap, N, seg + before + (sc[t] - cnt), status);
     }
-    if (t == 0 && rank == ranks - 1) *n_seg = before + total;
+    // (malformed offsets, flagged, can make more segments than their users size
+    // buffers for)
+    if (t == 0 && rank == ranks - 1) *n_seg = (int)min((long long)(before + total), segment_bound(N, n_lanes, cap));
 }
 
 __global__ void __cluster_dims__(PACK_BLOCKS, 1, 1) __launch_bounds__(BUILD_THREADS)

@@ -42,3 +42,25 @@ def test_more_scenarios_than_chunks(api, shape):
     ctx.check_status()
     for a, b in zip(got, ref):
         assert torch.equal(a, b)
+
+
+def test_malformed_offsets_past_the_window_are_flagged(api):
+    """Offsets that go back and forth make more segments than lanes of so few
+    vehicles can: the call flags them and leaves the context usable."""
+    L, K = 4000, 264
+    rng = np.random.default_rng(8)
+    sc = synth.make_scene([1, 2], rng)
+    dev = lambda x, t=torch.float32: torch.as_tensor(np.ascontiguousarray(x), dtype=t, device="cuda")  # noqa: E731
+    args = dev(sc["theta_true"]), dev(sc["p_init"]), dev(sc["v_init"])
+    y = torch.zeros((K, 3), device="cuda")
+    bad = api.Scene.from_lane_off(dev(np.arange(L + 1) % 2, torch.int32), dev(sc["length"]))
+    good = api.Scene.from_lane_off(dev(sc["lane_off"], torch.int32), dev(sc["length"]))
+    ctx = api.Context(vpt=4, warps_per_segment=4)
+    ref = api.loss_grad(*args, good, K, DT, y, 1, ctx=ctx)
+    ctx.check_status()
+    api.loss_grad(*args, bad, K, DT, y, 1, ctx=ctx)
+    with pytest.raises(Exception, match="lane"):
+        ctx.check_status()
+    for a, b in zip(api.loss_grad(*args, good, K, DT, y, 1, ctx=ctx), ref):
+        assert torch.equal(a, b)
+    ctx.check_status()
