@@ -724,8 +724,9 @@ backward_kernel(SimArgs a)
 // Kernel variants of one (vehicles per thread, warps per segment) shape:
 // seeds from dense gradients or from targets, fused Adam or gradient output,
 // with or without the delta gradient, tape blocks (SUB), and the slot mapping
-// (consecutive with dense seeds and, where the caller says so, with Adam;
-// one pair per thread has one mapping).
+// (consecutive with dense seeds and, with Adam and 4 vehicles per thread, where
+// the caller says so; the two are one with 2, and the consecutive code then
+// serves Adam).
 template <int VPT, int GW, bool SUB>
 inline void *backward_fn_t(bool dense, bool adam, bool wd, bool consec)
 {
@@ -733,8 +734,8 @@ inline void *backward_fn_t(bool dense, bool adam, bool wd, bool consec)
         return wd ? (void *)backward_kernel<VPT, GW, true, false, true, SUB, true>
                   : (void *)backward_kernel<VPT, GW, true, false, false, SUB, true>;
     if (adam)
-        return consec || VPT == 2 ? (void *)backward_kernel<VPT, GW, false, true, false, SUB, true>
-                                  : (void *)backward_kernel<VPT, GW, false, true, false, SUB, VPT == 2>;
+        return VPT != 4 || !consec ? (void *)backward_kernel<VPT, GW, false, true, false, SUB, VPT == 2>
+                                   : (void *)backward_kernel<VPT, GW, false, true, false, SUB, VPT <= 4>;
     return wd ? (void *)backward_kernel<VPT, GW, false, false, true, SUB, false>
               : (void *)backward_kernel<VPT, GW, false, false, false, SUB, false>;
 }

@@ -95,9 +95,9 @@ fit_fused_kernel(SimArgs a, long long part_stride)
 template <int VPT, int GW>
 inline void *fused_fn_t(bool sub, bool consec)
 {
-    if (consec || VPT == 2)
-        return sub ? (void *)fit_fused_kernel<VPT, GW, true, true> : (void *)fit_fused_kernel<VPT, GW, false, true>;
-    return sub ? (void *)fit_fused_kernel<VPT, GW, true, VPT == 2> : (void *)fit_fused_kernel<VPT, GW, false, VPT == 2>;
+    if (VPT != 4 || !consec)
+        return sub ? (void *)fit_fused_kernel<VPT, GW, true, VPT == 2> : (void *)fit_fused_kernel<VPT, GW, false, VPT == 2>;
+    return sub ? (void *)fit_fused_kernel<VPT, GW, true, VPT <= 4> : (void *)fit_fused_kernel<VPT, GW, false, VPT <= 4>;
 }
 
 // The forward, adjoint and single-launch fit kernels of one shape, as the

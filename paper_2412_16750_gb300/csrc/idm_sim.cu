@@ -381,13 +381,23 @@ size_t forward_smem_bytes(int vpt, int G, int wpb)
     return (size_t)grp_ctrl_floats(G) * (wpb / G) * sizeof(float);
 }
 
-// The slot mapping of a fit's adjoint: a scene's vehicles four to a thread in a
-// row (2M x 1,000 at interval 50: 15.45 -> 15.22 ms per iteration); a batch's
-// interleaved, because its losses are reported per scenario, and a scenario's
-// FP32 partial sums by thread keep their grouping.  Loss and gradient without
-// Adam stay interleaved too (10,000 lanes of 2-200 vehicles, 301 steps: 2.23 ms
-// against 2.31).
-static bool consecutive_slots(const SimArgs &a) { return a.scen_tab == nullptr; }
+// The slot mapping of a fit's adjoint.  Interleaved, but for a scene's long
+// horizons with 4 vehicles per thread, whose tape rows are one 16-byte access
+// when a thread's vehicles follow one another (2M x 1,000 at interval 50: 15.45
+// -> 15.22 ms per iteration); its loads and stores of vehicles, checkpoints and
+// moments then touch four times the sectors, which short horizons do not earn
+// back (40 iterations of 20,000 lanes of 100 over 9 steps: 9.86 ms consecutive,
+// 9.18 interleaved; 200 steps 7.53 and 7.63 per three), and with 8 vehicles per
+// thread no horizon does (three of 700 lanes of 2,000 over 200 steps at interval
+// 50: 9.83 and 8.13 ms, 40 over 9 steps 11.1 and 7.96).  A batch's losses are
+// reported per scenario, and a scenario's FP32 partial sums by thread keep their
+// grouping; loss and gradient without Adam stay interleaved too (10,000 lanes of
+// 2-200 vehicles, 301 steps: 2.23 ms against 2.31).
+constexpr int CONSEC_MIN_STEPS = 256;
+static bool consecutive_slots(int vpt, const SimArgs &a)
+{
+    return vpt == 4 && a.scen_tab == nullptr && a.scen0.K >= CONSEC_MIN_STEPS;
+}
 
 // Adjoint variants of every shape live in idm_shape_v<V>_g<G>.cu (with
 // 4 vehicles per thread, segments of up to 4 warps run in 4-warp blocks and
@@ -442,7 +452,7 @@ cudaError_t launch_backward(int vpt, int G, bool dense_seed, bool adam, bool wan
 {
     if (dense_seed && adam) return cudaErrorInvalidValue;
     if (wpb > backward_max_warps(vpt, G) || wpb % G || a.tape_cols > TMEM_COLS) return cudaErrorInvalidValue;
-    void *fn = backward_fn_v(vpt, G, dense_seed, adam, want_delta && !adam, a.tape_T < a.C, consecutive_slots(a));
+    void *fn = backward_fn_v(vpt, G, dense_seed, adam, want_delta && !adam, a.tape_T < a.C, consecutive_slots(vpt, a));
     if (!fn) return cudaErrorInvalidValue;
     size_t smem = backward_smem_bytes(vpt, a.tape_T, G, wpb, a.bwd_pf != 0);
     cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -467,7 +477,7 @@ cudaError_t launch_fit_fused(int vpt, int G, const SimArgs &a, long long part_st
                              cudaStream_t st)
 {
     if (wpb > backward_max_warps(vpt, G) || wpb % G || a.tape_cols > TMEM_COLS) return cudaErrorInvalidValue;
-    void *fn = fused_fn_v(vpt, G, a.tape_T < a.C, consecutive_slots(a));
+    void *fn = fused_fn_v(vpt, G, a.tape_T < a.C, consecutive_slots(vpt, a));
     if (!fn) return cudaErrorInvalidValue;
     const size_t smem = backward_smem_bytes(vpt, a.tape_T, G, wpb, a.bwd_pf != 0);
     cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
