@@ -299,9 +299,11 @@ struct Sweep {
         }
     }
 
-    // The copies fill occupied slots only: empty ones of the target rows hold 0.
+    // The copies fill occupied slots only, so empty ones of the dense seeds' rows
+    // are set to 0 (a target row's become 0 when its seeds are recorded).
     __device__ __forceinline__ void clear_empty(float *tr, int rows) const
     {
+        if (!DENSE) return;
 #pragma unroll
         for (int p = 0; p < NP; ++p)
 #pragma unroll
