@@ -145,10 +145,11 @@ int idm_event_counts(idm_ctx_t *ctx, void *stream, uint64_t *gap_floor_hits, uin
  * that hold the longest lane: such a call is bound by the latency of each
  * step, not by throughput); ckpt_interval: steps between stored checkpoints of the adjoint
  * (1..64, default 8); warps_per_block: 1..16 (default 8; rounded to a
- * multiple of warps_per_segment; the adjoint takes at least four, because
- * tensor memory is addressed by groups of four warps, and caps it by its
- * tape in shared and tensor memory and by its register budget: 4 warps for
- * vpt 4 with segments of up to 4 warps, 8 otherwise).  The forward runs the same segments with 8
+ * multiple of warps_per_segment; the adjoint takes at least four where a call
+ * has that many warps of segments per SM, because tensor memory is addressed by
+ * groups of four warps, and caps it by its tape in shared and tensor memory and
+ * by its register budget: 4 warps for vpt 4 with segments of up to 4 warps, 8
+ * otherwise).  The forward runs the same segments with 8
  * vehicles per thread where the capacity allows (e.g. 8 x 2 warps for the
  * adjoint's 4 x 4). */
 int idm_set_tuning(idm_ctx_t *ctx, int vpt, int warps_per_segment, int ckpt_interval, int warps_per_block);

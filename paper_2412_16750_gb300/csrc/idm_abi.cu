@@ -93,16 +93,24 @@ unsigned long long *event_counters(idm_ctx *c)
     return reinterpret_cast<unsigned long long *>(static_cast<char *>(c->status.p) + STATUS_EVENTS_OFF);
 }
 
-// Segments of `cap` slots that N vehicles in L lanes (or L segments of a batch)
-// make, about: whole lanes of the mean length, at most 7/8 of the slots, and one
-// per lane chunk where the builder keeps all of them (launch_build_segments).
-static long long expected_segments(long long N, long long L, int cap)
+// Segments of `cap` slots that N vehicles in L lanes make, about: whole lanes of
+// the mean length, at most 7/8 of the slots, and one per lane chunk where the
+// packing makes as many as it can (lanes_per_chunk).
+static long long expected_segments(long long N, long long L, int cap, bool one_wave)
 {
     const long long full = (long long)cap * 7 / 8;
     const long long lanes = std::max<long long>(1, cap / std::max<long long>(1, N / std::max<long long>(1, L)));
     long long segs = std::max((N + full - 1) / full, (L + lanes - 1) / lanes);
-    if (N < 16 * L) segs = std::max<long long>(segs, idm::SEG_BUILD_CHUNKS);
+    const long long per = (L + idm::SEG_BUILD_CHUNKS - 1) / idm::SEG_BUILD_CHUNKS;
+    if (one_wave || N < 16 * L) segs = std::max(segs, (L + per - 1) / per);
     return std::max<long long>(1, std::min<long long>(L, segs));
+}
+
+// ... of a prepared call: L lanes of a scene, or the L segments of a batch.
+static long long call_segments(const idm_ctx *c, const Prep *P, int L)
+{
+    if (P->a.scen_tab) return std::max(L, 1);
+    return expected_segments(P->a.N_total, L, 32 * P->vpt * P->G, lanes_fit_one_wave(c, L, P->G));
 }
 
 int pick_shape(idm_ctx *c, int max_lane, long long n_vehicles, int n_lanes, int *vpt, int *G)
@@ -117,7 +125,7 @@ int pick_shape(idm_ctx *c, int max_lane, long long n_vehicles, int n_lanes, int 
         if (max_lane > 1024) g = 8;
         // up to two such segments per SM: 2 vehicles per thread x 8 warps (the
         // same slots), two of those blocks per SM
-        if (max_lane <= 512 && expected_segments(n_vehicles, n_lanes, 512) <= 2LL * c->n_sm) {
+        if (max_lane <= 512 && expected_segments(n_vehicles, n_lanes, 512, false) <= 2LL * c->n_sm) {
             v = 2;
             g = 8;
         }
@@ -271,7 +279,7 @@ void forward_shape(int vpt, int G, long long segs, int n_sm, int *vpt_f, int *G_
 
 int forward_grid(idm_ctx *c, Prep *P, int L)
 {
-    const long long segs = expected_segments(P->a.N_total, L, 32 * P->vpt * P->G);
+    const long long segs = call_segments(c, P, L);
     forward_shape(P->vpt, P->G, segs, c->n_sm, &P->vpt_f, &P->G_f);
     const int G = P->G_f;
     if (P->vpt_f == 8) {
@@ -364,7 +372,7 @@ int backward_grid(idm_ctx *c, Prep *P, bool dense, bool adam, bool want_delta, i
     int groups = std::max(1, std::min(std::max(c->wpb, 4) / G, (int)(smem_max / per_group)));
     groups = std::max(1, std::min(groups, idm::backward_max_warps(P->vpt, G) / G));
     // few segments: spread over the SMs (in blocks of whole quarters of warps)
-    int spread = (int)((expected_segments(P->a.N_total, L, 32 * P->vpt * G) + c->n_sm - 1) / c->n_sm);
+    int spread = (int)((call_segments(c, P, L) + c->n_sm - 1) / c->n_sm);
     if (spread * G > 4) spread = ((spread * G + 3) / 4 * 4 + G - 1) / G;
     groups = std::min(groups, spread);
     while (groups > 1 && idm::tape_columns(P->vpt, T, groups * G) > idm::TMEM_COLS) --groups;
