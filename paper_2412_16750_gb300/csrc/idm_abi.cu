@@ -345,12 +345,12 @@ int backward_grid(idm_ctx *c, Prep *P, bool dense, bool adam, bool want_delta, i
     // prefetching the next run doubles two stages; use it when it does not cost a
     // resident group per SM, and not for one run.  The shared memory it takes is
     // the L1's, through which a fit's short iterations read and write parameters
-    // and moments: they have more than three runs to prefetch for (two of fewer
-    // than 8 steps).  40 iterations of 20,000 lanes of 100 over 8, 9 and 17 steps:
-    // 7.17, 8.91 and 12.1 ms with it, 6.85, 8.68 and 11.7 without; three runs of 4
-    // steps of the same lanes 2.50 with it and 2.53 without.
+    // and moments, so they prefetch from six runs on (three of fewer than 8
+    // steps).  40 iterations of 20,000 lanes of 100 over 8, 9 and 17 steps: 7.17,
+    // 8.91 and 12.1 ms with it, 6.85, 8.68 and 11.7 without; ten over 40 steps
+    // 5.61 and 5.55, over three runs of 4 steps 2.50 and 2.53.
     const int runs = (P->k_max + T - 1) / T;
-    const bool pf = runs > (!adam ? 1 : (T >= 8 ? 3 : 2)) &&
+    const bool pf = runs > (!adam ? 1 : (T >= 8 ? 5 : 2)) &&
                     groups_per_sm(T, true) >= std::min(reg_cap, groups_per_sm(T, false));
     P->a.bwd_pf = pf ? 1 : 0;
     P->a.tape_T = T;
