@@ -61,30 +61,43 @@ __device__ __forceinline__ int folds_every(const SimArgs &a)
 // A warp reaches the 32 lanes of its quarter (warp index mod 4) only, so the
 // warps w, w + 4, ... of a block use consecutive column ranges.
 // ---------------------------------------------------------------------------
-// Tensor memory of the block's tapes: `cols` columns (a power of two >= 32),
-// allocated and freed by warp 0; every thread of the block calls both.
-__device__ __forceinline__ uint32_t tape_alloc(int cols)
+// Tensor memory of the block's tapes: `cols` columns (a power of two >= 32) and,
+// for two steps more than the 8 that 128 columns hold with 4 vehicles per thread,
+// `more` of them; allocated and freed by warp 0, every thread of the block calls
+// both.  A block keeps the permit to allocate until it has both parts, so one that
+// waits for its second waits for blocks that hold all of theirs.  Three blocks of
+// 160 columns fit an SM; as one power of two each would take 256.
+struct TapeMem {
+    uint32_t at;    // first column
+    uint32_t jump;  // from the end of the first part to the second
+};
+__device__ __forceinline__ TapeMem tape_alloc(int cols, int more)
 {
-    __shared__ uint32_t slot;
-    if (threadIdx.x < 32) tc::tmem_alloc((uint32_t)__cvta_generic_to_shared(&slot), (uint32_t)cols);
+    __shared__ uint32_t slot[2];
+    if (threadIdx.x < 32) {
+        tc::tmem_alloc_part((uint32_t)__cvta_generic_to_shared(slot), (uint32_t)cols);
+        if (more > 0) tc::tmem_alloc_part((uint32_t)__cvta_generic_to_shared(slot + 1), (uint32_t)more);
+        tc::tmem_alloc_done();
+    }
     tc::fence_before_sync();
     __syncthreads();
     tc::fence_after_sync();
-    return slot;
+    return TapeMem{slot[0], more > 0 ? slot[1] - slot[0] - (uint32_t)cols : 0u};
 }
-__device__ __forceinline__ void tape_free(uint32_t tmem, int cols)
+__device__ __forceinline__ void tape_free(TapeMem m, int cols, int more)
 {
     tc::fence_before_sync();
     __syncthreads();
     if (threadIdx.x < 32) {
         tc::fence_after_sync();
-        tc::tmem_dealloc(tmem, (uint32_t)cols);
+        if (more > 0) tc::tmem_dealloc(m.at + (uint32_t)cols + m.jump, (uint32_t)more);
+        tc::tmem_dealloc(m.at, (uint32_t)cols);
     }
 }
 // This warp's columns: `words` per warp, quarter warp mod 4 of the lanes.
-__device__ __forceinline__ uint32_t tape_base(uint32_t tmem, int warp, int words)
+__device__ __forceinline__ TapeMem tape_base(TapeMem m, int warp, int words)
 {
-    return tmem + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)((warp >> 2) * words);
+    return TapeMem{m.at + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)((warp >> 2) * words), m.jump};
 }
 
 __device__ __forceinline__ void tape_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
@@ -260,7 +273,7 @@ __device__ __forceinline__ void segment_epilogue(const SimArgs &a, const Seg &sg
 // row of targets or dense seeds that becomes the seeds (each [SLG] floats, the
 // lane's 2 NP slots adjacent), the tensor memory the other coefficients.
 // ---------------------------------------------------------------------------
-template <int NP, bool DENSE, bool WD, bool D4, bool CONSEC>
+template <int NP, bool DENSE, bool WD, bool D4, bool CONSEC, bool JUMP>
 struct Sweep {
     const SimArgs &a;
     const ScenDesc &sc;
@@ -273,7 +286,7 @@ struct Sweep {
     const int wl;         // scenario-local index of this lane's first slot
     const int TS;         // floats of T tape rows
     float *const tv;      // this lane's slots of the speed row 0; frd rows TS after
-    const uint32_t tape;  // tensor-memory column of step 0
+    const TapeMem tape;   // tensor memory of the recorded steps
     f2 lp[NP], lv[NP];    // adjoints of position and speed
     f2 sacc[6][NP];       // the six factored gradient sums, over all steps
     f2 qc[NP];            // 4 a_max / v0 (D4)
@@ -282,7 +295,7 @@ struct Sweep {
     int xp = 0, fp = 0;   // parities of the exchange cells
 
     __device__ __forceinline__ Sweep(const SimArgs &a_, const ScenDesc &sc_, const Seg &sg, int lb, Grp &g_, float *base,
-                                     uint32_t tape_, int T, const VehConst2 (&kc_)[NP], State2 (&st_)[NP])
+                                     TapeMem tape_, int T, const VehConst2 (&kc_)[NP], State2 (&st_)[NP])
         : a(a_), sc(sc_), g(g_), kc(kc_), st(st_), SLG(64 * NP * g_.G), wb(g_.w * 64 * NP),
           at0(g_.w * 64 * NP + pair_slot<NP, CONSEC>(0, g_.lane)), wl(lb + at0), TS(T * 64 * NP * g_.G),
           tv(base + at0), tape(tape_)
@@ -297,6 +310,14 @@ struct Sweep {
 #pragma unroll
             for (int q = 0; q < 6; ++q) sacc[q][p] = F2(0.0f);
         }
+    }
+
+    // Tensor-memory column of recorded step s from its column in one part (JUMP:
+    // from the ninth step on in the second; the others skip the arithmetic, which
+    // costs 2 %).
+    __device__ __forceinline__ uint32_t column(uint32_t at, int s) const
+    {
+        return JUMP ? at + (uint32_t)(s >> 3) * tape.jump : at;
     }
 
     // The copies fill occupied slots only, so empty ones of the dense seeds' rows
@@ -480,21 +501,21 @@ struct Sweep {
         {
             int obs_k = first_obs(c0), k = c0;
             float *rv = tv, *rr = tr;
-            uint32_t at = tape;
+            uint32_t at = tape.at;
             for (int s = 0; s + 1 < n; ++s, ++k, rv += SLG, rr += SLG, at += TAPE_WORDS * 2 * NP) {
                 const bool obs = k == obs_k;
                 if (!DENSE && k == split) {
                     lfirst = lseg;
                     lseg = F2(0.0f);
                 }
-                record(true, obs, rv, rr, at, scale, lseg);
+                record(true, obs, rv, rr, column(at, s), scale, lseg);
                 obs_k += obs ? sc.obs_stride : 0;
             }
             if (!DENSE && k == split) {
                 lfirst = lseg;
                 lseg = F2(0.0f);
             }
-            record(end, k == obs_k, rv, rr, at, scale, lseg);
+            record(end, k == obs_k, rv, rr, column(at, n - 1), scale, lseg);
         }
         if (end) {  // the state is now at step K: seed of the final step
             if (DENSE) {
@@ -520,13 +541,13 @@ struct Sweep {
         grp_sync(g);  // the whole group's tape is written
         Rec J;
         const float *rv = tv + (n - 1) * SLG, *rr = tr + (n - 1) * SLG;
-        uint32_t at = tape + (uint32_t)((n - 1) * TAPE_WORDS * 2 * NP);
-        read(rv, at, J);
+        uint32_t at = tape.at + (uint32_t)((n - 1) * TAPE_WORDS * 2 * NP);
+        read(rv, column(at, n - 1), J);
         int k = c0 + n - 1;
         for (int s = n - 1; s >= 1; --s, --k, rr -= SLG) {
             rv -= SLG;
             at -= TAPE_WORDS * 2 * NP;
-            reverse<true>(J, rr, k, rv, at);
+            reverse<true>(J, rr, k, rv, column(at, s - 1));
         }
         reverse<false>(J, rr, k, rv, at);
     }
@@ -546,10 +567,10 @@ struct Sweep {
 // segment, last first.
 template <int NP, bool DENSE, bool ADAM, bool WD, bool D4, bool CONSEC>
 __device__ __forceinline__ void backward_segment(const SimArgs &a, const ScenDesc &sc, const Seg &sg, int s_idx, int lb,
-                                                 Grp &g, float *base, uint32_t tape, const VehConst2 (&kc)[NP],
+                                                 Grp &g, float *base, TapeMem tape, const VehConst2 (&kc)[NP],
                                                  State2 (&st)[NP])
 {
-    Sweep<NP, DENSE, WD, D4, CONSEC> w(a, sc, sg, lb, g, base, tape, a.C, kc, st);
+    Sweep<NP, DENSE, WD, D4, CONSEC, false> w(a, sc, sg, lb, g, base, tape, a.C, kc, st);
     const int nb = a.bwd_pf ? 2 : 1;                     // stages (two with prefetch)
     float *trb = w.tv + bwd_target_row(a.C, nb > 1) * w.SLG;  // nb target tapes
     float *ckb = nb > 1 ? trb + nb * w.TS : w.tv;        // checkpoint stage [STATE_ROWS][SLG] (without prefetch over the tape)
@@ -578,26 +599,27 @@ __device__ __forceinline__ void backward_segment(const SimArgs &a, const ScenDes
     w.template finish<ADAM>(sg, s_idx);
 }
 
-// The same adjoint when the tape is shallower than the checkpoint interval:
+// The same adjoint when the tape is shallower than the checkpoint interval, or
+// has a second part of tensor memory (an interval of 9 or 10 steps in one run):
 // each checkpoint segment is first run forward once writing sub-checkpoints
 // every T steps (global scratch, this thread's own slots), then processed as
 // tape blocks of T steps, last first.
 template <int NP, bool DENSE, bool ADAM, bool WD, bool D4, bool CONSEC>
 __device__ __forceinline__ void backward_segment_blocks(const SimArgs &a, const ScenDesc &sc, const Seg &sg, int s_idx,
-                                                        int lb, Grp &g, float *base, uint32_t tape,
+                                                        int lb, Grp &g, float *base, TapeMem tape,
                                                         const VehConst2 (&kc)[NP], State2 (&st)[NP])
 {
     const int T = a.tape_T;
-    Sweep<NP, DENSE, WD, D4, CONSEC> w(a, sc, sg, lb, g, base, tape, T, kc, st);
+    Sweep<NP, DENSE, WD, D4, CONSEC, NP == 2> w(a, sc, sg, lb, g, base, tape, T, kc, st);
     const int nb = a.bwd_pf ? 2 : 1;
     float *trb = w.tv + bwd_target_row(T, nb > 1) * w.SLG;
     float *ckb = nb > 1 ? trb + nb * w.TS : w.tv;
     w.clear_empty(trb, nb * T);
     // Block j > 0 of a checkpoint segment starts from sub-checkpoint row j - 1,
     // block 0 from the checkpoint.  With several vehicle pairs per thread (tapes
-    // of 8 steps) the first block takes the remainder: the forward pass then
-    // ends where the last full block begins (42 steps of 50 instead of 48: two
-    // iterations of 2M x 1,000 31.13 -> 30.89 ms).
+    // of 8 or 10 steps) the first block takes the remainder: the forward pass then
+    // ends where the last full block begins (42 steps of 50 instead of 48 with
+    // tapes of 8: two iterations of 2M x 1,000 31.13 -> 30.89 ms).
     constexpr bool SHORT_FIRST = NP >= 2;
     auto seg_len = [&](int cs) { return min(a.C, sc.K - cs * a.C); };
     auto n_sub = [&](int cs) { return (seg_len(cs) + T - 1) / T; };
@@ -669,10 +691,13 @@ __device__ __forceinline__ void backward_segment_blocks(const SimArgs &a, const 
     w.template finish<ADAM>(sg, s_idx);
 }
 
-// Register budgets: 2 vehicles per thread fit 128 registers (2 blocks of 8
-// warps per SM); 4 per thread need ~168 without spilling, so their blocks
-// are 4 warps (3 blocks per SM) unless the segment has 8 warps (256 threads,
-// one block per SM); 8 per thread use up to 255.
+// Register budgets: 2 vehicles per thread fit 128 registers (2 blocks of 8 warps
+// per SM); 4 per thread take 168, so their blocks are 4 warps (3 blocks per SM)
+// unless the segment has 8 warps (256 threads, one block per SM); 8 per thread use
+// up to 255.  Some of what stays live across a step's barriers spills: up to 36
+// bytes with 4 per thread, up to 200 with 8 (the delta gradient with tape blocks).
+// The same loops bounded to one block of twelve warps (as many registers) came
+// out 2 to 4 % slower.
 template <int VPT, int GW>
 struct BwdBounds {
     static constexpr bool narrow = VPT == 4 && GW < 8;
@@ -695,8 +720,8 @@ backward_kernel(SimArgs a)
     float *gbase = smem + (warp / G) * bwd_group_floats(VPT, a.tape_T, G, a.bwd_pf != 0);
     float *ctrl = gbase + bwd_group_floats(VPT, a.tape_T, G, a.bwd_pf != 0) - grp_ctrl_floats(G);
     Grp g = make_grp(G, ctrl);
-    const uint32_t tmem = tape_alloc(a.tape_cols);
-    const uint32_t tape = tape_base(tmem, warp, TAPE_WORDS * VPT * a.tape_T);
+    const TapeMem tmem = tape_alloc(a.tape_cols, VPT == 4 && SUB ? a.tape_more : 0);
+    const TapeMem tape = tape_base(tmem, warp, TAPE_WORDS * VPT * a.tape_T);
     int par = 0;
     for (;;) {
         const int s_idx = grp_next(g, a.work, par);
@@ -720,7 +745,7 @@ backward_kernel(SimArgs a)
                 backward_segment<NP, DENSE, ADAM, WD, false, CONSEC>(a, sc, sg, s_idx, lb, g, gbase, tape, kc, st);
         }
     }
-    tape_free(tmem, a.tape_cols);
+    tape_free(tmem, a.tape_cols, VPT == 4 && SUB ? a.tape_more : 0);
 }
 
 // Kernel variants of one (vehicles per thread, warps per segment) shape:

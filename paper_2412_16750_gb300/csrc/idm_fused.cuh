@@ -44,8 +44,8 @@ fit_fused_kernel(SimArgs a, long long part_stride)
         if (threadIdx.x == 0) atomicOr(a.status, IDM_STATUS_LANE_TOO_LONG);
         return;
     }
-    const uint32_t tmem = tape_alloc(a.tape_cols);
-    const uint32_t tape = tape_base(tmem, warp, TAPE_WORDS * VPT * a.tape_T);
+    const TapeMem tmem = tape_alloc(a.tape_cols, VPT == 4 && SUB ? a.tape_more : 0);
+    const TapeMem tape = tape_base(tmem, warp, TAPE_WORDS * VPT * a.tape_T);
     double *const part0 = a.loss_part;
     const FwdFlags ff{false, false, true, false};
     int par = 0;
@@ -89,7 +89,7 @@ fit_fused_kernel(SimArgs a, long long part_stride)
             grp_sync(g);  // and the adjoint's last reads before the next forward's first writes
         }
     }
-    tape_free(tmem, a.tape_cols);
+    tape_free(tmem, a.tape_cols, VPT == 4 && SUB ? a.tape_more : 0);
 }
 
 template <int VPT, int GW>

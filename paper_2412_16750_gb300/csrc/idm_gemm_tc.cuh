@@ -198,11 +198,19 @@ __device__ __forceinline__ void tma_load_2d(uint32_t dst, const void *tmap, int 
 }
 
 // Whole-warp tensor-memory allocation; the address is written to shared memory.
-__device__ __forceinline__ void tmem_alloc(uint32_t dst_smem, uint32_t ncols)
+__device__ __forceinline__ void tmem_alloc_part(uint32_t dst_smem, uint32_t ncols)
 {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(dst_smem), "r"(ncols)
                  : "memory");
+}
+__device__ __forceinline__ void tmem_alloc_done()
+{
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void tmem_alloc(uint32_t dst_smem, uint32_t ncols)
+{
+    tmem_alloc_part(dst_smem, ncols);
+    tmem_alloc_done();
 }
 
 __device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t ncols)

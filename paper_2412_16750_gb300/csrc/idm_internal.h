@@ -59,7 +59,8 @@ struct SimArgs {
     int C;                      // checkpoint interval (steps)
     int loss_split;             // > 0: the horizon's one run sums the loss of the steps before it apart
     int tape_T;                 // adjoint tape depth (steps, <= C); tape_T < C uses sub_ckpt
-    int tape_cols;              // tensor-memory columns of an adjoint block's tapes
+    int tape_cols;              // tensor-memory columns of an adjoint block's tapes,
+    int tape_more;              // and of their steps from the ninth on (backward_narrow; else 0)
     float *sub_ckpt;            // [ceil(C/tape_T)-1][STATE_ROWS][N_total] states inside a checkpoint segment
     unsigned *status;
     // adjoint
@@ -129,6 +130,10 @@ size_t forward_smem_bytes(int vpt, int G, int wpb);
 // Largest adjoint block (warps) for a shape: 4 for 4 vehicles per thread in
 // segments of up to 4 warps (register budget), else 8.
 int backward_max_warps(int vpt, int G);
+// 4 vehicles per thread in segments of up to 4 warps: three blocks of four warps
+// per SM, each with 128 columns for 8 steps of tape or 32 more for 10.
+bool backward_narrow(int vpt, int G);
+constexpr int NARROW_STEPS = 8, NARROW_STEPS_MORE = 10, NARROW_COLS_MORE = 32;
 // Adjoint warps per SM the register budgets allow for a shape.
 int backward_resident_warps(int vpt, int G);
 // max_part: at least the number of partials (n_seg * per_seg).

@@ -399,6 +399,10 @@ static bool consecutive_slots(int vpt, const SimArgs &a)
     return vpt == 4 && a.scen_tab == nullptr && a.scen0.K >= CONSEC_MIN_STEPS;
 }
 
+// The kernels with tape blocks: for a tape shallower than the interval, and for
+// one with a second part.
+static bool tape_blocks(const SimArgs &a) { return a.tape_T < a.C || a.tape_more > 0; }
+
 // Adjoint variants of every shape live in idm_shape_v<V>_g<G>.cu (with
 // 4 vehicles per thread, segments of up to 4 warps run in 4-warp blocks and
 // 8-warp segments in 8-warp blocks); SUB: tape shallower than the checkpoint
@@ -438,12 +442,14 @@ int backward_blocks_per_sm(int vpt, int G, bool dense, bool adam, bool want_delt
     return fn ? adjoint_blocks_per_sm(fn, G, wpb, smem, cols) : 1;
 }
 
-int backward_max_warps(int vpt, int G) { return (vpt == 4 && G <= 4) ? 4 : 8; }
+bool backward_narrow(int vpt, int G) { return vpt == 4 && G <= 4; }
+
+int backward_max_warps(int vpt, int G) { return backward_narrow(vpt, G) ? 4 : 8; }
 
 int backward_resident_warps(int vpt, int G)
 {
     if (vpt == 2) return 16;
-    if (vpt == 4 && G <= 4) return 12;
+    if (backward_narrow(vpt, G)) return 12;
     return 8;
 }
 
@@ -451,8 +457,8 @@ cudaError_t launch_backward(int vpt, int G, bool dense_seed, bool adam, bool wan
                             int wpb, cudaStream_t st)
 {
     if (dense_seed && adam) return cudaErrorInvalidValue;
-    if (wpb > backward_max_warps(vpt, G) || wpb % G || a.tape_cols > TMEM_COLS) return cudaErrorInvalidValue;
-    void *fn = backward_fn_v(vpt, G, dense_seed, adam, want_delta && !adam, a.tape_T < a.C, consecutive_slots(vpt, a));
+    if (wpb > backward_max_warps(vpt, G) || wpb % G || a.tape_cols + a.tape_more > TMEM_COLS) return cudaErrorInvalidValue;
+    void *fn = backward_fn_v(vpt, G, dense_seed, adam, want_delta && !adam, tape_blocks(a), consecutive_slots(vpt, a));
     if (!fn) return cudaErrorInvalidValue;
     size_t smem = backward_smem_bytes(vpt, a.tape_T, G, wpb, a.bwd_pf != 0);
     cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -476,8 +482,8 @@ static void *fused_fn_v(int vpt, int G, bool sub, bool consec)
 cudaError_t launch_fit_fused(int vpt, int G, const SimArgs &a, long long part_stride, int grid, int wpb,
                              cudaStream_t st)
 {
-    if (wpb > backward_max_warps(vpt, G) || wpb % G || a.tape_cols > TMEM_COLS) return cudaErrorInvalidValue;
-    void *fn = fused_fn_v(vpt, G, a.tape_T < a.C, consecutive_slots(vpt, a));
+    if (wpb > backward_max_warps(vpt, G) || wpb % G || a.tape_cols + a.tape_more > TMEM_COLS) return cudaErrorInvalidValue;
+    void *fn = fused_fn_v(vpt, G, tape_blocks(a), consecutive_slots(vpt, a));
     if (!fn) return cudaErrorInvalidValue;
     const size_t smem = backward_smem_bytes(vpt, a.tape_T, G, wpb, a.bwd_pf != 0);
     cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -485,7 +491,7 @@ cudaError_t launch_fit_fused(int vpt, int G, const SimArgs &a, long long part_st
     int dev = 0, n_sm = 1;
     if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
     if ((e = cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-    const int cap = n_sm * adjoint_blocks_per_sm(fn, G, wpb, smem, a.tape_cols);
+    const int cap = n_sm * adjoint_blocks_per_sm(fn, G, wpb, smem, a.tape_cols + a.tape_more);
     SimArgs args = a;
     args.G = G;
     long long stride = part_stride;
