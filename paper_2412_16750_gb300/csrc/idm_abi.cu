@@ -339,18 +339,27 @@ int backward_grid(idm_ctx *c, Prep *P, bool dense, bool adam, bool want_delta, i
         return fail(c, IDM_ERR_ARG, "adjoint tape does not fit shared memory for vpt %d x %d warps", P->vpt, G);
     P->a.sub_ckpt = nullptr;
     if (T < C) {
-        const size_t rows = (size_t)((C + T - 1) / T - 1);
-        const int rc = ensure(c, c->sub_ckpt, sizeof(float) * idm::STATE_ROWS * rows * (size_t)std::max(P->a.N_total, 1),
-                              "sub-checkpoints");
-        // no room for them: an interval that fits the chip as one tape runs so,
-        // with fewer groups per SM
-        if (rc == IDM_ERR_WORKSPACE && idm::tape_columns(P->vpt, C, G) <= idm::TMEM_COLS && groups_per_sm(C, false) > 0) {
-            T = C;
-            more = false;
-        } else if (rc)
-            return rc;
-        else
-            P->a.sub_ckpt = (float *)c->sub_ckpt.p;
+        auto rows = [&](int t) { return (C + t - 1) / t - 1; };
+        auto take = [&](int t) {
+            return ensure(c, c->sub_ckpt,
+                          sizeof(float) * idm::STATE_ROWS * (size_t)rows(t) * (size_t)std::max(P->a.N_total, 1),
+                          "sub-checkpoints");
+        };
+        int rc = take(T);
+        // no room for them: a deeper tape with fewer of them, or none, that still
+        // fits the chip, with fewer groups per SM
+        for (int t = T + 1, r = rows(T); rc == IDM_ERR_WORKSPACE && t <= C; ++t) {
+            if (idm::tape_columns(P->vpt, t, G) > idm::TMEM_COLS || groups_per_sm(t, false) == 0) break;
+            if (rows(t) == r) continue;
+            r = rows(t);
+            rc = r > 0 ? take(t) : IDM_OK;
+            if (rc == IDM_OK) {
+                T = t;
+                more = false;
+            }
+        }
+        if (rc) return rc;
+        if (T < C) P->a.sub_ckpt = (float *)c->sub_ckpt.p;
     }
     // prefetching the next run doubles two stages; use it when it does not cost a
     // resident group per SM, and not for one run.  The shared memory it takes is
