@@ -304,7 +304,7 @@ def adjoint_roofline(N, K, ckpt, bwd_avg_ms, n_sm, peaks, peak_kind):
         "sfu": {"ops_per_vehicle_step": ADJ_SFU_PER_VS, "achieved": sfu_achieved, "peak": sfu_peak,
                 "frac": sfu_achieved / sfu_peak, "unit": "G special-function ops/s",
                 "peak_source": "nominal: %d SMs x %d per clock x %.0f MHz" % (n_sm, SFU_PER_SM_CLK, sm_mhz)},
-        "hbm_achieved_gbs": (4.0 + 16.0 / ckpt) * units / t / 1e9,
+        "hbm_achieved_gbs": (4.0 + 20.0 / ckpt) * units / t / 1e9,
         "hbm_peak_gbs": peaks.get("hbm_gbs"),
     }
 
@@ -1068,7 +1068,7 @@ def run_gpu(a, rank, world, local_rank):
                  "roofline": adjoint_roofline(N, K, a.tuned_ckpt, mt["bwd_avg_ms"], n_sm, peaks, peak_kind),
                  "note": "the same workload with the checkpoint interval whose adjoint tape fits the chip "
                          "(no tape blocks); checkpoints then take %.1f GB instead of %.2f GB"
-                         % (16.0 * N * math.ceil(K / a.tuned_ckpt) / 1e9, 16.0 * N * math.ceil(K / a.ckpt) / 1e9)}
+                         % (20.0 * N * math.ceil(K / a.tuned_ckpt) / 1e9, 20.0 * N * math.ceil(K / a.ckpt) / 1e9)}
         ctx.set_tuning(a.vpt, a.G, a.ckpt, a.wpb)
 
     # ---- Sec. III-C events of the fitted and the true parameters ------------

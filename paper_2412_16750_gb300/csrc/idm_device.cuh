@@ -64,8 +64,6 @@ __device__ __forceinline__ f2 ex2(f2 x) { return make_float2(ex2_approx(x.x), ex
 __device__ __forceinline__ f2 lg2(f2 x) { return make_float2(lg2_approx(x.x), lg2_approx(x.y)); }
 __device__ __forceinline__ f2 rcp2(f2 x) { return make_float2(rcp_approx(x.x), rcp_approx(x.y)); }
 __device__ __forceinline__ f2 vmax(f2 a, f2 b) { return make_float2(fmaxf(a.x, b.x), fmaxf(a.y, b.y)); }
-__device__ __forceinline__ f2 vabs(f2 a) { return make_float2(fabsf(a.x), fabsf(a.y)); }
-
 __device__ __forceinline__ f2 neg2(f2 a) { return make_float2(-a.x, -a.y); }
 
 // Softplus pieces: e = exp(-|x|) = 2^(-|x| log2 e) and

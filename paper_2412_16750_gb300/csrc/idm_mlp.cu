@@ -756,7 +756,7 @@ __global__ void __launch_bounds__(FEAT_THREADS) features_kernel(const FeatArgs f
     const bool ok = i >= 0 && i < f.N;
     live[threadIdx.x] = ok;
     if (ok) {
-        const bool head = is_lane_head(f.lane_off, f.n_lanes, i);
+        const bool head = i == 0 || is_lane_head(f.lane_off, f.n_lanes, i);  // (offsets may not start at 0)
         const float inv_2sdt = 1.0f / (2.0f * (float)f.obs_stride * f.dt);
         const float y0 = f.p_init[i];
         uint32_t *out = stage[threadIdx.x];

@@ -1331,8 +1331,8 @@ extern "C" int idm_recon_fit(idm_ctx_t *c, const idm_recon_t *r, idm_params_t *p
         a.hi[q] = box_hi[q];
     }
     if (loss_hist) IDM_CK(cudaMemsetAsync(loss_hist, 0, sizeof(double) * n_iter, st));
-    // Two blocks per SM leave shared memory for copies two chunks ahead (97 KB),
-    // three for one (75 KB): measured per iteration on GB300, 6,101
+    // Two blocks per SM leave shared memory for copies two chunks ahead (88.7 KB
+    // a block), three for one (72.3 KB): measured per iteration on GB300, 6,101
     // trajectories (191 blocks) 128 and 131 us, 21,750 (680 blocks) 280 and
     // 261 us, 12,000 170 and 162 us.
     if ((a.N + 31) / 32 <= 2 * c->n_sm)

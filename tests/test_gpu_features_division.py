@@ -63,3 +63,14 @@ def test_rows_equal_true_division(api, kind, origin):
     assert torch.equal(got.isnan(), nan)
     same = (got.view(torch.int16) == ref.view(torch.int16)) | nan
     assert bool(same.all()), (int((~same).sum()), got[~same][:4], ref[~same][:4])
+
+
+def test_first_vehicle_has_no_vehicle_before_it(api):
+    """Offsets that do not start at 0 (malformed) leave vehicle 0 in no lane: its
+    rows are those of a lane head, and nothing in front of the arrays is read."""
+    rng = np.random.default_rng(0)
+    cuda = lambda x: torch.as_tensor(np.asarray(x, np.float32), device="cuda")  # noqa: E731
+    args = cuda(rng.normal(0, 100, 5)), cuda(rng.normal(20, 3, 5)), 20, 0.1, cuda(rng.normal(0, 100, (PREFIX, 5)))
+    rows = [api.mlp_features(api.Scene.from_lane_off(torch.tensor(off, dtype=torch.int32), torch.full((5,), 5.0)), *args)
+            for off in ([0, 1, 5], [1, 3, 5])]
+    assert torch.equal(rows[0][0], rows[1][0])
