@@ -113,7 +113,7 @@ static long long call_segments(const idm_ctx *c, const Prep *P, int L)
     return expected_segments(P->a.N_total, L, 32 * P->vpt * P->G, lanes_fit_one_wave(c, L, P->G));
 }
 
-int pick_shape(idm_ctx *c, int max_lane, long long n_vehicles, int n_lanes, int *vpt, int *G)
+int pick_shape(idm_ctx *c, int max_lane, long long n_vehicles, int n_lanes, long long least_segs, int *vpt, int *G)
 {
     int v = c->vpt_req, g = c->G_req;
     if (v == 0 && g == 0) {
@@ -125,7 +125,8 @@ int pick_shape(idm_ctx *c, int max_lane, long long n_vehicles, int n_lanes, int 
         if (max_lane > 1024) g = 8;
         // up to two such segments per SM: 2 vehicles per thread x 8 warps (the
         // same slots), two of those blocks per SM
-        if (max_lane <= 512 && expected_segments(n_vehicles, n_lanes, 512, false) <= 2LL * c->n_sm) {
+        if (max_lane <= 512 &&
+            std::max(expected_segments(n_vehicles, n_lanes, 512, false), least_segs) <= 2LL * c->n_sm) {
             v = 2;
             g = 8;
         }
@@ -198,7 +199,7 @@ static int prepare(idm_ctx *c, const idm_scene_t *sc, const idm_params_t *pr, co
             const idm_sim_t *sim, bool need_ckpt, bool need_loss, int obs_stride, Prep *P, cudaStream_t st)
 {
     int rc;
-    if ((rc = pick_shape(c, sc->max_lane, sc->n_vehicles, sc->n_lanes, &P->vpt, &P->G))) return rc;
+    if ((rc = pick_shape(c, sc->max_lane, sc->n_vehicles, sc->n_lanes, 0, &P->vpt, &P->G))) return rc;
     const int N = sc->n_vehicles, L = sc->n_lanes;
     const int G = P->G;
     if ((rc = ensure(c, c->seg, sizeof(Seg) * (size_t)L, "segments"))) return rc;

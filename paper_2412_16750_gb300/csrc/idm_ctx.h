@@ -80,8 +80,9 @@ constexpr size_t STATUS_EVENTS_OFF = 16;
 unsigned long long *event_counters(idm_ctx *c);
 // Kernel shape for a call: the context's request, else 4 x 4 (8 x 4, 8 x 8
 // for longer lanes), or for a scene that fits one wave of 2-vehicle warps
-// the latency shape 2 x G.
-int pick_shape(idm_ctx *c, int max_lane, long long n_vehicles, int n_lanes, int *vpt, int *G);
+// the latency shape 2 x G.  least_segs: segments of 512 slots that a batch's
+// scenarios make at least (a scene: 0).
+int pick_shape(idm_ctx *c, int max_lane, long long n_vehicles, int n_lanes, long long least_segs, int *vpt, int *G);
 // Every lane as a segment of its own of G warps fits one wave of 16 warps per SM.
 bool lanes_fit_one_wave(const idm_ctx *c, int n_lanes, int G);
 // Forward shape for the segment capacity of the adjoint shape (vpt, G) and

@@ -126,7 +126,7 @@ extern "C" int idm_loss_grad_noalloc(const idm_scene_t *sc, const idm_params_t *
         cudaDeviceGetAttribute(&c.n_sm, cudaDevAttrMultiProcessorCount, c.device) != cudaSuccess)
         return IDM_ERR_CUDA;
     Prep P;
-    if ((rc = pick_shape(&c, sc->max_lane, sc->n_vehicles, sc->n_lanes, &P.vpt, &P.G))) return rc;
+    if ((rc = pick_shape(&c, sc->max_lane, sc->n_vehicles, sc->n_lanes, 0, &P.vpt, &P.G))) return rc;
     const size_t N = (size_t)sc->n_vehicles, L = (size_t)sc->n_lanes;
     const int G = P.G;
     const int C = std::min(c.C, sim->K);  // as idm_loss_grad: at most the horizon
