@@ -20,19 +20,18 @@ namespace idm {
 // gradient sums of each slot accumulate in registers and are folded into
 // compensated totals about every FOLD_STEPS steps.
 //
-// The coefficients come out of the recompute's own model evaluation (they
-// share its softplus, reciprocal and power terms; the reverse sweep used to
-// evaluate them again from the recorded speed and gap).  Four of them per
+// The coefficients come out of the recompute's own model evaluation, whose
+// softplus, reciprocal and power terms they share.  Four of them per
 // vehicle go to tensor memory: private to the thread that reads them back, 64
 // KB per SM quarter that a kernel without matrix products leaves idle, and
 // beside the shared memory that the tape of speeds, seeds and the fifth
 // coefficient, and the next run's copies, fill to the last resident block.
-// Bound by issue and dependent latency (ncu on 500,000 vehicles x 200 steps:
-// 56 % of the issue slots, FMA pipe 48 % of its cycles, DRAM 10 %; 419
-// warp-instructions per warp and step with the delta gradient).  Measured on
-// GB300 with the same packing, two evaluations -> one: loss + gradient of 10,000
-// uneven lanes over 301 steps 2.35 -> 2.2 ms, of 1,500 lanes of 100 over 300
-// steps 542 -> 432 us; a 50-iteration fit of 1,000 vehicles 3.10 -> 2.78 ms.
+// Bound by issue and dependent latency (ncu on 400,000 vehicles x 256 steps:
+// 57 % of the issue slots, FMA pipe 46 % of its cycles, 3.31 warp-instructions
+// per vehicle and step).  Measured on GB300 with the same packing, against a
+// second evaluation in the reverse sweep: loss + gradient of 10,000 uneven lanes
+// over 301 steps 2.35 -> 2.2 ms, of 1,500 lanes of 100 over 300 steps 542 -> 432
+// us; a 50-iteration fit of 1,000 vehicles 3.08 -> 2.82 ms.
 // ---------------------------------------------------------------------------
 // Compensated gradient sums.  Within a fold window of max(1, FOLD_STEPS / C)
 // checkpoint segments (counted from the last) the six factored sums of a slot
@@ -663,7 +662,7 @@ __device__ __forceinline__ void backward_segment_blocks(const SimArgs &a, const 
 #pragma unroll
                 for (int p = 0; p < NP; ++p) {
                     const bool x = w.mask[p][0] != 0, y = w.mask[p][1] != 0;
-                const int o = pair_off<CONSEC>(p);
+                    const int o = pair_off<CONSEC>(p);
                     store_pair(row, o, st[p].ph, x, y);
                     store_pair(row + m, o, st[p].pl, x, y);
                     store_pair(row + 2 * m, o, st[p].v, x, y);
